@@ -313,7 +313,8 @@ vplbm_status vplbm_group_step(vplbm_solver* const* solvers, int32_t n,
                               const int64_t* steps);
 
 /* Kernel launches this solver issued on its hot path (fused steps and mask
- * updates) since creation. */
+ * updates; the sums of step records, one per up to 64 steps of a call, are not
+ * counted) since creation. */
 int64_t vplbm_launch_count(const vplbm_solver* s);
 
 /* Timing of the fused step kernel: enable = 1 brackets each fused launch with
@@ -355,7 +356,7 @@ vplbm_status vplbm_fused_timing(vplbm_solver* s, double* total_ms, int64_t* laun
  *  flag      device int set to 1 if the step produced rho <= 0 or a
  *            non-finite velocity (never cleared here), or NULL.
  *
- * Scratch: the per-tile and per-group reduction sums live in a fixed 1 MiB
+ * Scratch: the per-tile and per-chunk reduction sums live in a fixed 1 MiB
  * device array inside the library, which every GPU that loads the library
  * holds until the process exits. It holds at most 43,491 tiles of the fused
  * step: with tiles of 128 x 32 nodes (FP32 and 16-bit storage) about 178.1M

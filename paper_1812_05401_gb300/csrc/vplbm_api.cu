@@ -23,6 +23,7 @@
 #include "vplbm.h"
 #include "vplbm_launch.h"
 #include "vplbm_params.h"
+#include "vplbm_reduce.cuh"
 
 using namespace vplbm;
 
@@ -143,6 +144,28 @@ __global__ void perturbation_kernel(double* u, int nx, int ny, double u0x, doubl
   u[nn + node] = amp > 0.0 ? __dadd_rn(u0y, r2[1]) : u0y;
 }
 
+// Step records of one solver: block (step, chunk).
+__global__ void __launch_bounds__(kThreads) reduce_kernel(const __grid_constant__ ReduceArgs a) {
+  __shared__ double sm[kThreads / 32][3];
+  __shared__ int s_last;
+  reduce_steps(a, blockIdx.x, blockIdx.y, sm, &s_last);
+}
+
+// Step records of a group's window starting at the group's step k0: block
+// (member * kWindow + step, chunk). Members list their whole group call
+// (t0 and steps of the call).
+__global__ void __launch_bounds__(kThreads)
+    reduce_group_kernel(const ReduceArgs* __restrict__ members, long long k0) {
+  __shared__ double sm[kThreads / 32][3];
+  __shared__ int s_last;
+  ReduceArgs a = members[blockIdx.x / kWindow];
+  const int step = blockIdx.x % kWindow;
+  a.steps = min((long long)kWindow, a.steps - k0);
+  a.t0 += k0;
+  if (step >= a.steps || int(blockIdx.y) >= reduce_chunks(a.n_tiles)) return;
+  reduce_steps(a, step, blockIdx.y, sm, &s_last);
+}
+
 dim3 grid2d(int w, int h, dim3 blk) {
   return dim3((w + blk.x - 1) / blk.x, (h + blk.y - 1) / blk.y);
 }
@@ -177,9 +200,9 @@ struct vplbm_solver {
   int cur = 0;  // buffer holding f*(t)
   uint8_t* mask = nullptr;
   void* us = nullptr;
-  double* partials = nullptr;
-  double* group_partials = nullptr;
-  unsigned* counters = nullptr;
+  double* partials = nullptr;    // [kWindow][n_tiles][3]
+  double* chunk_sums = nullptr;  // [kWindow][n_chunks][3]
+  unsigned* counters = nullptr;  // [kWindow]
   double* ring = nullptr;
   int* flag = nullptr;
   int* static_box = nullptr;  // device box {x0, y0, x1, y1} of the static solid layer
@@ -198,7 +221,7 @@ struct vplbm_solver {
   int64_t me_read = 0;  // first step not yet returned by vplbm_momentum_exchange_forces
   int64_t me_stop = 0;  // step at which recording last stopped
 
-  int tiles_x = 0, tiles_y = 0, n_tiles = 0, n_groups = 0;
+  int tiles_x = 0, tiles_y = 0, n_tiles = 0;
   StepParams base{};  // constants; src/dst/t/bodies filled per step
 
   int64_t t = 0;
@@ -590,6 +613,25 @@ StepParams step_params(const vplbm_solver* s, int64_t t, int parity) {
   return p;
 }
 
+ReduceArgs reduce_args(const vplbm_solver* s, int64_t t0, int64_t steps) {
+  ReduceArgs a{};
+  a.partials = s->partials;
+  a.chunk_sums = s->chunk_sums;
+  a.counters = s->counters;
+  a.ring = s->ring;
+  a.t0 = t0;
+  a.n_tiles = s->n_tiles;
+  a.steps = steps;
+  a.ring_len = s->cfg.force_ring_len;
+  a.reduce_mass = s->base.reduce_mass;
+  return a;
+}
+
+cudaError_t launch_reduce(const ReduceArgs& a, cudaStream_t st) {
+  reduce_kernel<<<dim3(unsigned(a.steps), reduce_chunks(a.n_tiles)), kThreads, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_fused(const vplbm_solver* s, const StepParams& p) {
   const int coll = p.collision;
   switch (s->cfg.storage) {
@@ -728,14 +770,19 @@ int tile_rows_of(const vplbm_config* c) {
   return rows;
 }
 
-void tiles_of(const vplbm_config* c, int* tx, int* ty, int* nt, int* ng) {
+void tiles_of(const vplbm_config* c, int* tx, int* ty, int* nt) {
   const int tw = tile_x(c->storage);
   const int rows = tile_rows_of(c);
   *tx = (c->nx + tw - 1) / tw;
   *ty = (c->ny + rows - 1) / rows;
   *nt = *tx * *ty;
-  *ng = (*nt + kGroup - 1) / kGroup;
 }
+
+// Reduction scratch of a solver: a window of tile partials, their chunk sums
+// and the arrival counters.
+size_t partials_bytes(int nt) { return 3 * sizeof(double) * size_t(kWindow) * size_t(nt); }
+size_t chunk_sums_bytes(int nt) { return 3 * sizeof(double) * size_t(kWindow) * size_t(reduce_chunks(nt)); }
+size_t counters_bytes() { return sizeof(unsigned) * size_t(kWindow); }
 
 vplbm_status check_usable(vplbm_solver* s) {
   if (!s) return VPLBM_ERR_INVALID;
@@ -796,16 +843,15 @@ double vplbm_tau_from_reynolds(double u_ref, double l_ref, double re) {
 size_t vplbm_footprint_bytes(const vplbm_config* c) {
   std::string why;
   if (validate(c, &why) != VPLBM_OK) return 0;
-  int tx, ty, nt, ng;
-  tiles_of(c, &tx, &ty, &nt, &ng);
+  int tx, ty, nt;
+  tiles_of(c, &tx, &ty, &nt);
   const size_t pitch = size_t(row_pitch(c->nx, c->storage));
   const size_t plane = pitch * size_t(c->ny);
   const bool aa = c->streaming == VPLBM_STREAM_AA;
   size_t b = (aa ? 1 : 2) * 9 * plane * element_size(c->storage);  // A/B or in-place populations
   if (aa && c->bc_x != VPLBM_BC_PERIODIC) b += 9 * size_t(c->ny) * element_size(c->storage);
   b += plane;                                            // mask
-  b += 3 * sizeof(double) * (size_t(nt) + size_t(ng));   // reduction partials
-  b += sizeof(unsigned) * (size_t(ng) + 1);
+  b += partials_bytes(nt) + chunk_sums_bytes(nt) + counters_bytes();  // reduction scratch
   b += 3 * sizeof(double) * size_t(c->force_ring_len);
   b += sizeof(int) + sizeof(kEmptyBox);                  // error flag, static solid box
   if (c->bc_x == VPLBM_BC_INLET_CONVECTIVE) b += 2 * 3 * size_t(c->ny) * ghost_elem(c->storage);
@@ -835,7 +881,7 @@ vplbm_status vplbm_create(const vplbm_config* cfg, vplbm_solver** out) {
   s->esize = element_size(cfg->storage);
   s->pitch = row_pitch(cfg->nx, cfg->storage);
   s->plane = (long long)s->pitch * cfg->ny;
-  tiles_of(cfg, &s->tiles_x, &s->tiles_y, &s->n_tiles, &s->n_groups);
+  tiles_of(cfg, &s->tiles_x, &s->tiles_y, &s->n_tiles);
 
   auto bail = [&](vplbm_status st) {
     std::fprintf(stderr, "vplbm_create: %s\n", s->err.c_str());
@@ -858,16 +904,16 @@ vplbm_status vplbm_create(const vplbm_config* cfg, vplbm_solver** out) {
   if ((st = mem_get(s, &s->f[0], pop)) != VPLBM_OK ||
       (!s->aa && (st = mem_get(s, &s->f[1], pop)) != VPLBM_OK) ||
       (st = mem_get(s, &s->mask, size_t(s->plane))) != VPLBM_OK ||
-      (st = mem_get(s, &s->partials, 3 * sizeof(double) * s->n_tiles)) != VPLBM_OK ||
-      (st = mem_get(s, &s->group_partials, 3 * sizeof(double) * s->n_groups)) != VPLBM_OK ||
-      (st = mem_get(s, &s->counters, sizeof(unsigned) * (s->n_groups + 1))) != VPLBM_OK ||
+      (st = mem_get(s, &s->partials, partials_bytes(s->n_tiles))) != VPLBM_OK ||
+      (st = mem_get(s, &s->chunk_sums, chunk_sums_bytes(s->n_tiles))) != VPLBM_OK ||
+      (st = mem_get(s, &s->counters, counters_bytes())) != VPLBM_OK ||
       (st = mem_get(s, &s->ring, 3 * sizeof(double) * cfg->force_ring_len)) != VPLBM_OK ||
       (st = mem_get(s, &s->flag, sizeof(int))) != VPLBM_OK ||
       (st = mem_get(s, &s->static_box, sizeof(kEmptyBox))) != VPLBM_OK) {
     return bail(st);
   }
   if ((e = cudaMemsetAsync(s->mask, 0, size_t(s->plane), s->stream)) != cudaSuccess ||
-      (e = cudaMemsetAsync(s->counters, 0, sizeof(unsigned) * (s->n_groups + 1), s->stream)) != cudaSuccess ||
+      (e = cudaMemsetAsync(s->counters, 0, counters_bytes(), s->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(s->ring, 0, 3 * sizeof(double) * cfg->force_ring_len, s->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(s->flag, 0, sizeof(int), s->stream)) != cudaSuccess ||
       (e = cudaMemcpyAsync(s->static_box, kEmptyBox, sizeof(kEmptyBox), cudaMemcpyHostToDevice,
@@ -912,11 +958,7 @@ vplbm_status vplbm_create(const vplbm_config* cfg, vplbm_solver** out) {
   p.lost = s->lost;
   physics_consts(cfg, &p);
   p.partials = s->partials;
-  p.group_partials = s->group_partials;
-  p.counters = s->counters;
-  p.ring = s->ring;
   p.flag = s->flag;
-  p.ring_len = cfg->force_ring_len;
   p.reduce_mass = cfg->reduce_mass ? 1 : 0;
   p.stochastic = cfg->rounding == VPLBM_ROUND_STOCHASTIC ? 1 : 0;
 
@@ -1019,9 +1061,11 @@ vplbm_status vplbm_step(vplbm_solver* s, int64_t n) {
   if (st != VPLBM_OK) return st;
   if (n < 0) return fail(s, VPLBM_ERR_INVALID, "n must be >= 0");
   TraceRange trace("vplbm_step");
+  int64_t window = 0;  // steps whose tile partials await their sum
   for (int64_t k = 0; k < n; ++k) {
     if ((st = ensure_mask(s, s->t)) != VPLBM_OK) return st;
-    const StepParams p = step_params(s, s->t, 0);
+    StepParams p = step_params(s, s->t, 0);
+    p.partials += 3 * (long long)s->n_tiles * window;
     if (s->me_on) {
       VP_CUDA(s, launch_momentum_exchange(s, p, s->me_ring + 2 * (s->t % s->cfg.force_ring_len)));
       s->launches++;
@@ -1040,6 +1084,10 @@ vplbm_status vplbm_step(vplbm_solver* s, int64_t n) {
     s->launches++;
     s->cur ^= 1;
     s->t++;
+    if (++window == kWindow || k == n - 1) {
+      VP_CUDA(s, launch_reduce(reduce_args(s, s->t - window, window), s->stream));
+      window = 0;
+    }
   }
   return VPLBM_OK;
 }
@@ -1445,6 +1493,8 @@ vplbm_status vplbm_group_step(vplbm_solver* const* solvers, int32_t n, const int
     int cls = 0;
     StepParams* d_params = nullptr;
     GroupTile* d_table = nullptr;
+    ReduceArgs* d_reduce = nullptr;
+    int max_chunks = 1;
     std::vector<int64_t> prefix_steps;  // steps of the j-th member (descending)
     std::vector<int> prefix_tiles;      // tiles of members 0..j
   };
@@ -1457,6 +1507,7 @@ vplbm_status vplbm_group_step(vplbm_solver* const* solvers, int32_t n, const int
       for (auto& pl : v) {
         if (pl.d_params) cudaFreeAsync(pl.d_params, stream);
         if (pl.d_table) cudaFreeAsync(pl.d_table, stream);
+        if (pl.d_reduce) cudaFreeAsync(pl.d_reduce, stream);
       }
     }
   } owned{{}, stream};
@@ -1469,6 +1520,7 @@ vplbm_status vplbm_group_step(vplbm_solver* const* solvers, int32_t n, const int
                        [](const Member& a, const Member& b) { return a.steps > b.steps; });
       std::vector<StepParams> hp;
       std::vector<GroupTile> ht;
+      std::vector<ReduceArgs> hr;
       plans.emplace_back();
       Plan& pl = plans.back();
       pl.storage = sg;
@@ -1478,11 +1530,16 @@ vplbm_status vplbm_group_step(vplbm_solver* const* solvers, int32_t n, const int
         hp.push_back(step_params(s, s->t, 0));
         hp.push_back(step_params(s, s->t, 1));
         for (int tile = 0; tile < s->n_tiles; ++tile) ht.push_back(GroupTile{int(j), tile});
+        hr.push_back(reduce_args(s, s->t, mem[j].steps));
+        pl.max_chunks = std::max(pl.max_chunks, reduce_chunks(s->n_tiles));
         pl.prefix_steps.push_back(mem[j].steps);
         pl.prefix_tiles.push_back(int(ht.size()));
       }
       VP_CUDA(s0, cudaMallocAsync(reinterpret_cast<void**>(&pl.d_params), hp.size() * sizeof(StepParams), stream));
       VP_CUDA(s0, cudaMallocAsync(reinterpret_cast<void**>(&pl.d_table), ht.size() * sizeof(GroupTile), stream));
+      VP_CUDA(s0, cudaMallocAsync(reinterpret_cast<void**>(&pl.d_reduce), hr.size() * sizeof(ReduceArgs), stream));
+      VP_CUDA(s0, cudaMemcpyAsync(pl.d_reduce, hr.data(), hr.size() * sizeof(ReduceArgs),
+                                  cudaMemcpyHostToDevice, stream));
       VP_CUDA(s0, cudaMemcpyAsync(pl.d_params, hp.data(), hp.size() * sizeof(StepParams),
                                   cudaMemcpyHostToDevice, stream));
       VP_CUDA(s0, cudaMemcpyAsync(pl.d_table, ht.data(), ht.size() * sizeof(GroupTile),
@@ -1499,6 +1556,14 @@ vplbm_status vplbm_group_step(vplbm_solver* const* solvers, int32_t n, const int
       const int mode = pl.cls == 0 ? kModeAB
                                    : (((pl.cls - 1) ^ int(k & 1)) == 0 ? kModeAAPush : kModeAALocal);
       VP_CUDA(s0, launch_group(pl.storage, pl.d_params, pl.d_table, nb, k, mode, stream));
+      // the records of a full window, or of the plan's last steps
+      if (k % kWindow == kWindow - 1 || k == pl.prefix_steps[0] - 1) {
+        const int64_t k0 = k - k % kWindow;
+        int members = 0;  // those with a step in this window (a prefix)
+        while (members < int(pl.prefix_steps.size()) && pl.prefix_steps[members] > k0) ++members;
+        reduce_group_kernel<<<dim3(members * kWindow, pl.max_chunks), kThreads, 0, stream>>>(pl.d_reduce, k0);
+        VP_CUDA(s0, cudaGetLastError());
+      }
     }
     for (int i : moving) {
       if (steps[i] > k) {
@@ -1567,7 +1632,7 @@ void vplbm_destroy(vplbm_solver* s) {
   }
   for (auto e : s->ev_pool) cudaEventDestroy(e);
   if (s->stream) {
-    void* bufs[] = {s->f[0], s->aa ? nullptr : s->f[1], s->mask, s->us, s->partials, s->group_partials,
+    void* bufs[] = {s->f[0], s->aa ? nullptr : s->f[1], s->mask, s->us, s->partials, s->chunk_sums,
                     s->counters, s->ring, s->flag, s->static_box, s->me_ring,
                     s->me_scratch, s->me_counter, s->ghost[0], s->ghost[1], s->z, s->lost};
     if (s->cfg.dev_free) cudaStreamSynchronize(s->stream);  // once, for all of them
@@ -1592,14 +1657,14 @@ void vplbm_destroy(vplbm_solver* s) {
 // step: code running inside a CUDA graph being built, a host callback, a
 // real-time loop with a fixed memory budget, or a framework that owns every
 // allocation itself. The reduction scratch of the fused step (per-tile and
-// per-group partial sums and the arrival counters) lives in the fixed array
+// per-chunk partial sums and the arrival counters) lives in the fixed array
 // below instead of per-solver cudaMalloc'd buffers. Every GPU that loads this
 // library holds the array until the process exits.
 // ===========================================================================
 
 namespace {
 
-// 1 MiB: 24 bytes per tile, 24 per group of 256 tiles, 4 per group counter
+// 1 MiB: 24 bytes per tile, 24 per slot of 256 tiles, 4 per slot's counter
 // (+1), 16-byte alignment and the 4-byte flag hold at most 43,491 tiles.
 constexpr size_t kNoAllocScratchBytes = size_t(1) << 20;
 
@@ -1610,15 +1675,21 @@ constexpr int kNoAllocMaxDevices = 64;
 std::mutex g_noalloc_mutex;
 void* g_noalloc_addr[kNoAllocMaxDevices] = {nullptr};
 
-// Byte layout of the scratch for n_tiles tiles: partials, group partials,
+// Tiles that share one slot of chunk sums and counters in the scratch's
+// layout; it fixes the largest grid the scratch takes (a step needs one slot
+// per kChunkTiles tiles, so there are more than enough).
+constexpr int kNoAllocSlotTiles = 256;
+static_assert(kNoAllocSlotTiles <= kChunkTiles, "one slot of chunk sums per chunk");
+
+// Byte layout of the scratch for n_tiles tiles: partials, chunk sums,
 // counters, divergence flag. Returns the bytes used.
-size_t noalloc_layout(int n_tiles, size_t* off_group, size_t* off_counters, size_t* off_flag) {
-  const int n_groups = (n_tiles + kGroup - 1) / kGroup;
+size_t noalloc_layout(int n_tiles, size_t* off_chunks, size_t* off_counters, size_t* off_flag) {
+  const int n_slots = (n_tiles + kNoAllocSlotTiles - 1) / kNoAllocSlotTiles;
   size_t off = 3 * sizeof(double) * size_t(n_tiles);
-  *off_group = off;
-  off += 3 * sizeof(double) * size_t(n_groups);
+  *off_chunks = off;
+  off += 3 * sizeof(double) * size_t(n_slots);
   *off_counters = off;
-  off += sizeof(unsigned) * size_t(n_groups + 1);
+  off += sizeof(unsigned) * size_t(n_slots + 1);
   off = (off + 15) & ~size_t(15);
   *off_flag = off;
   off += sizeof(int);
@@ -1660,10 +1731,10 @@ extern "C" vplbm_status vplbm_step_noalloc(const vplbm_config* cfg, const vplbm_
                          "state between steps (use vplbm_create / vplbm_step)\n");
     return VPLBM_ERR_INVALID;
   }
-  int tx, ty, nt, ng;
-  tiles_of(cfg, &tx, &ty, &nt, &ng);
-  size_t off_group, off_counters, off_flag;
-  const size_t need = noalloc_layout(nt, &off_group, &off_counters, &off_flag);
+  int tx, ty, nt;
+  tiles_of(cfg, &tx, &ty, &nt);
+  size_t off_chunks, off_counters, off_flag;
+  const size_t need = noalloc_layout(nt, &off_chunks, &off_counters, &off_flag);
   if (need > kNoAllocScratchBytes) {
     std::fprintf(stderr,
                  "vplbm_step_noalloc: grid of %d x %d needs %zu bytes of reduction scratch; the "
@@ -1746,11 +1817,7 @@ extern "C" vplbm_status vplbm_step_noalloc(const vplbm_config* cfg, const vplbm_
     }
   }
   p.partials = reinterpret_cast<double*>(sb);
-  p.group_partials = reinterpret_cast<double*>(sb + off_group);
-  p.counters = reinterpret_cast<unsigned*>(sb + off_counters);
   p.flag = flag ? flag : reinterpret_cast<int*>(sb + off_flag);
-  p.ring = record;  // one record: ring of length 1
-  p.ring_len = 1;
   p.reduce_mass = cfg->reduce_mass ? 1 : 0;
   p.stochastic = cfg->rounding == VPLBM_ROUND_STOCHASTIC ? 1 : 0;
   p.t = t;
@@ -1760,6 +1827,19 @@ extern "C" vplbm_status vplbm_step_noalloc(const vplbm_config* cfg, const vplbm_
     case kF32: e = launch_fused_f32(p.collision, p, stream); break;
     case kF16: e = launch_fused_f16(p.collision, p, stream); break;
     default: e = launch_fused_bf16(p.collision, p, stream); break;
+  }
+  if (e == cudaSuccess) {
+    ReduceArgs a{};
+    a.partials = p.partials;
+    a.chunk_sums = reinterpret_cast<double*>(sb + off_chunks);
+    a.counters = reinterpret_cast<unsigned*>(sb + off_counters);
+    a.ring = record;  // one record: ring of length 1
+    a.t0 = t;
+    a.n_tiles = nt;
+    a.steps = 1;
+    a.ring_len = 1;
+    a.reduce_mass = p.reduce_mass;
+    e = launch_reduce(a, stream);
   }
   if (e != cudaSuccess) {
     std::fprintf(stderr, "vplbm_step_noalloc: launch: %s\n", cudaGetErrorString(e));

@@ -19,6 +19,7 @@
 #include <type_traits>
 
 #include "vplbm_params.h"
+#include "vplbm_reduce.cuh"
 
 namespace vplbm {
 
@@ -610,125 +611,6 @@ __device__ __forceinline__ void collide_mrt(const StepParams& p, T h[9], const M
 }
 
 // ---------------------------------------------------------------------------
-// Deterministic block and grid reductions in FP64.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Sum of v[0..2] over the block of NT threads, fixed order; result valid in
-// thread 0.
-template <int NT = kThreads>
-__device__ __forceinline__ void block_sum3(double v[3], double (*sm)[3]) {
-  const int tid = threadIdx.x + threadIdx.y * blockDim.x;
-  constexpr int n_warps = NT / 32;
-  const int lane = tid & 31, warp = tid >> 5;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) v[k] = warp_sum(v[k]);
-  if (lane == 0) {
-    sm[warp][0] = v[0];
-    sm[warp][1] = v[1];
-    sm[warp][2] = v[2];
-  }
-  __syncthreads();
-  if (tid == 0) {
-    for (int k = 0; k < 3; ++k) {
-      double s = 0.0;
-      for (int w = 0; w < n_warps; ++w) s += sm[w][k];
-      v[k] = s;
-    }
-  }
-  __syncthreads();
-}
-
-// Finishes the per-step reduction once this tile's partial is written: the
-// last tile of each group of kGroup tiles sums the group in tile order, and
-// the last group to finish sums the groups in group order and writes the
-// step's record (a grid of a single group writes its group sum directly).
-// Both levels are fixed-order, so the result does not depend on which blocks
-// ran when.
-template <int NT>
-__device__ __forceinline__ void finish_reduction(const StepParams& p, int tile, long long t,
-                                                 const double tile_sum[3], double (*sm)[3]) {
-  __shared__ int s_last;
-  const int tid = threadIdx.x + threadIdx.y * blockDim.x;
-  constexpr int n_threads = NT;
-  const int group = tile / kGroup;
-  const int n_groups = (p.n_tiles + kGroup - 1) / kGroup;
-  if (tid == 0) {
-    double* dst = p.partials + 3ll * tile;
-    __stcg(dst + 0, tile_sum[0]);
-    __stcg(dst + 1, tile_sum[1]);
-    __stcg(dst + 2, tile_sum[2]);
-    __threadfence();
-    const int gsize = min(kGroup, p.n_tiles - group * kGroup);
-    const unsigned prev = atomicAdd(p.counters + group, 1u);
-    s_last = (prev == (unsigned)(gsize - 1));
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  {
-    double v[3] = {0.0, 0.0, 0.0};
-    const int t0 = group * kGroup;
-    const int gsize = min(kGroup, p.n_tiles - t0);
-    // each thread adds its strided share of the group's tiles in increasing
-    // order (one tile per thread for 8-warp blocks, two for 4-warp blocks)
-    for (int i = tid; i < gsize; i += n_threads) {
-      const double* src = p.partials + 3ll * (t0 + i);
-      v[0] += __ldcg(src + 0);
-      v[1] += __ldcg(src + 1);
-      v[2] += __ldcg(src + 2);
-    }
-    block_sum3<NT>(v, sm);
-    if (tid == 0) {
-      p.counters[group] = 0u;  // ready for the next step
-      if (n_groups == 1) {
-        // one group (a small grid): its sum is the step's record
-        double* r = p.ring + 3ll * (t % p.ring_len);
-        r[0] = v[0];
-        r[1] = v[1];
-        r[2] = p.reduce_mass ? v[2] : 0.0;
-        s_last = 0;
-      } else {
-        double* g = p.group_partials + 3ll * group;
-        __stcg(g + 0, v[0]);
-        __stcg(g + 1, v[1]);
-        __stcg(g + 2, v[2]);
-        __threadfence();
-        const unsigned prev = atomicAdd(p.counters + n_groups, 1u);
-        s_last = (prev == (unsigned)(n_groups - 1));
-      }
-    }
-    __syncthreads();
-  }
-  if (!s_last) return;
-  __threadfence();
-  double v[3] = {0.0, 0.0, 0.0};
-  for (int g = tid; g < n_groups; g += n_threads) {
-    // each thread adds its strided share in increasing group order
-    v[0] += __ldcg(p.group_partials + 3ll * g + 0);
-    v[1] += __ldcg(p.group_partials + 3ll * g + 1);
-    v[2] += __ldcg(p.group_partials + 3ll * g + 2);
-  }
-  block_sum3<NT>(v, sm);
-  if (tid == 0) {
-    double* r = p.ring + 3ll * (t % p.ring_len);
-    r[0] = v[0];
-    r[1] = v[1];
-    r[2] = p.reduce_mass ? v[2] : 0.0;
-    p.counters[n_groups] = 0u;
-  }
-}
-
-// ---------------------------------------------------------------------------
 // The fused time step of one tile: (32 N) x tile_y nodes, N = npt(STORE). Lane
 // l of warp w takes nodes x0 + N l .. x0 + N l + N - 1 of rows y0 + w + W r,
 // r = 0..rows_per_warp-1, W = warps_per_block(STORE).
@@ -1029,7 +911,8 @@ __device__ __forceinline__ typename S::E fstar_e(const StepParams& p, const type
 // MODE: kModeAB (pull from p.src, store to p.dst), or one of the two in-place
 // AA steps on the one buffer p.dst (== p.src).
 template <int STORE, int COLL, int MODE = kModeAB>
-__device__ __forceinline__ void step_tile(const StepParams& p, int tile, long long t) {
+__device__ __forceinline__ void step_tile(const StepParams& p, int tile, long long t,
+                                          double* partials) {
   using S = Store<STORE>;
   using T = typename S::T;
   using E = typename S::E;
@@ -1238,8 +1121,8 @@ __device__ __forceinline__ void step_tile(const StepParams& p, int tile, long lo
     sm[warp][1] = bfy;
   }
   const int block_solid = __syncthreads_or(any_solid);
-  double ts[3] = {0.0, 0.0, 0.0};
   if (tid == 0) {
+    double ts[3] = {0.0, 0.0, 0.0};
     T msum = T(0);
 #pragma unroll
     for (int w = 0; w < W; ++w) msum += smass[w];
@@ -1255,15 +1138,18 @@ __device__ __forceinline__ void step_tile(const StepParams& p, int tile, long lo
       const int nact = min(TX, p.nx - x0) * min(p.tile_y, p.ny - y0);
       ts[2] = double(nact) + double(msum);
     }
+    // the tile's share of the step's record; reduce_kernel adds the tiles
+    double* out = partials + 3ll * tile;
+    out[0] = ts[0];
+    out[1] = ts[1];
+    out[2] = ts[2];
   }
-  __syncthreads();
-  finish_reduction<threads_per_block(STORE)>(p, tile, t, ts, sm);
 }
 
 template <int STORE, int COLL, int MODE = kModeAB>
 __global__ void __launch_bounds__(threads_per_block(STORE), min_blocks_per_sm(STORE))
     fused_step_kernel(const __grid_constant__ StepParams p) {
-  step_tile<STORE, COLL, MODE>(p, blockIdx.x, p.t);
+  step_tile<STORE, COLL, MODE>(p, blockIdx.x, p.t, p.partials);
 }
 
 // Grouped launch for serving: block b runs tile table[b].tile of solver
@@ -1290,10 +1176,11 @@ __global__ void __launch_bounds__(threads_per_block(STORE), min_blocks_per_sm(ST
       to[w] = __ldg(from + w);
   }
   __syncthreads();
+  double* partials = sp.partials + 3ll * sp.n_tiles * (k % kWindow);
   if (sp.collision == kTrt)
-    step_tile<STORE, kTrt, MODE>(sp, gt.tile, sp.t + k);
+    step_tile<STORE, kTrt, MODE>(sp, gt.tile, sp.t + k, partials);
   else
-    step_tile<STORE, kMrt, MODE>(sp, gt.tile, sp.t + k);
+    step_tile<STORE, kMrt, MODE>(sp, gt.tile, sp.t + k, partials);
 }
 
 // ---------------------------------------------------------------------------

@@ -60,7 +60,14 @@ __host__ __device__ constexpr int tile_x(int storage) { return kLanes * npt(stor
 // Block shape of the per-node kernels (initialisation, moments, import/export).
 constexpr int kBlockX = 64;
 constexpr int kBlockY = 4;
-constexpr int kGroup = 256;             // tiles per first-level reduction group
+// The fused step leaves one partial (F_x, F_y, sum rho) per tile; one launch
+// adds the partials of up to kWindow steps. Tiles beyond kChunkTiles are added
+// by several blocks (8 per step for 16384 x 4096).
+constexpr int kWindow = 64;
+constexpr int kChunkTiles = 2048;
+__host__ __device__ constexpr int reduce_chunks(int n_tiles) {
+  return (n_tiles + kChunkTiles - 1) / kChunkTiles;
+}
 constexpr int kMeBlocks = 304;          // fixed grid of the momentum-exchange reduction (2 per SM)
 constexpr uint8_t kStaticSolid = 255;   // mask value of a node solid through the static mask
 
@@ -114,13 +121,9 @@ struct StepParams {
   long long plane;          // pitch * ny
   Consts<double> cd;        // constants for the FP64 kernels
   Consts<float> cf;         // the same, rounded, for the FP32 kernels
-  double* partials;         // [n_tiles][3]
-  double* group_partials;   // [n_groups][3]
-  unsigned* counters;       // [n_groups + 1], zero between steps
-  double* ring;             // [ring_len][3]: F_x, F_y, sum rho per step
+  double* partials;         // [n_tiles][3] of this step (grouped: [kWindow][n_tiles][3])
   int* flag;                // set to 1 on divergence
   long long t;              // index of this step
-  int ring_len;
   int reduce_mass;
   int stochastic;           // 16-bit stores: 1 = stochastic rounding, 0 = nearest even
   int collision;            // kTrt | kMrt (read by the grouped kernel)
@@ -139,6 +142,17 @@ template <> __host__ __device__ inline const Consts<float>& consts<float>(const 
 struct GroupTile {
   int solver;
   int tile;
+};
+
+// Arguments of the sum of a window's tile partials into the step records.
+struct ReduceArgs {
+  const double* partials;  // [steps][n_tiles][3]
+  double* chunk_sums;      // [kWindow][reduce_chunks(n_tiles)][3] (more than one chunk)
+  unsigned* counters;      // [kWindow], zero between launches
+  double* ring;            // [ring_len][3]: F_x, F_y, sum rho per step
+  long long t0;            // step index of the window's first step
+  long long steps;         // steps of the window (grouped: of the member's whole call)
+  int n_tiles, ring_len, reduce_mass;
 };
 
 // Arguments of the momentum-exchange reduction: a box of candidate solid
