@@ -47,6 +47,8 @@ struct BodyGeomSet {
 // outcome is reproducible.
 __global__ void mask_update_kernel(uint8_t* mask, int pitch, int x0, int y0, int w, int h,
                                    const __grid_constant__ BodyGeomSet g) {
+  pdl_trigger();
+  pdl_wait();
   const int x = x0 + blockIdx.x * blockDim.x + threadIdx.x;
   const int y = y0 + blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= x0 + w || y >= y0 + h) return;
@@ -148,6 +150,8 @@ __global__ void perturbation_kernel(double* u, int nx, int ny, double u0x, doubl
 __global__ void __launch_bounds__(kThreads) reduce_kernel(const __grid_constant__ ReduceArgs a) {
   __shared__ double sm[kThreads / 32][3];
   __shared__ int s_last;
+  pdl_trigger();
+  pdl_wait();
   reduce_steps(a, blockIdx.x, blockIdx.y, sm, &s_last);
 }
 
@@ -158,6 +162,8 @@ __global__ void __launch_bounds__(kThreads)
     reduce_group_kernel(const ReduceArgs* __restrict__ members, long long k0) {
   __shared__ double sm[kThreads / 32][3];
   __shared__ int s_last;
+  pdl_trigger();
+  pdl_wait();
   ReduceArgs a = members[blockIdx.x / kWindow];
   const int step = blockIdx.x % kWindow;
   a.steps = min((long long)kWindow, a.steps - k0);
@@ -397,9 +403,8 @@ vplbm_status launch_mask_update(vplbm_solver* s, Box box, int64_t t) {
   }
   const dim3 blk(64, 4);
   const int w = box.x1 - box.x0 + 1, h = box.y1 - box.y0 + 1;
-  mask_update_kernel<<<grid2d(w, h, blk), blk, 0, s->stream>>>(s->mask, s->pitch, box.x0, box.y0, w,
-                                                               h, g);
-  VP_CUDA(s, cudaGetLastError());
+  VP_CUDA(s, launch_pdl(mask_update_kernel, grid2d(w, h, blk), blk, s->stream, s->mask, s->pitch, box.x0,
+                        box.y0, w, h, g));
   s->launches++;
   return VPLBM_OK;
 }
@@ -628,8 +633,7 @@ ReduceArgs reduce_args(const vplbm_solver* s, int64_t t0, int64_t steps) {
 }
 
 cudaError_t launch_reduce(const ReduceArgs& a, cudaStream_t st) {
-  reduce_kernel<<<dim3(unsigned(a.steps), reduce_chunks(a.n_tiles)), kThreads, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(reduce_kernel, dim3(unsigned(a.steps), reduce_chunks(a.n_tiles)), dim3(kThreads), st, a);
 }
 
 cudaError_t launch_fused(const vplbm_solver* s, const StepParams& p) {
@@ -1561,8 +1565,8 @@ vplbm_status vplbm_group_step(vplbm_solver* const* solvers, int32_t n, const int
         const int64_t k0 = k - k % kWindow;
         int members = 0;  // those with a step in this window (a prefix)
         while (members < int(pl.prefix_steps.size()) && pl.prefix_steps[members] > k0) ++members;
-        reduce_group_kernel<<<dim3(members * kWindow, pl.max_chunks), kThreads, 0, stream>>>(pl.d_reduce, k0);
-        VP_CUDA(s0, cudaGetLastError());
+        VP_CUDA(s0, launch_pdl(reduce_group_kernel, dim3(members * kWindow, pl.max_chunks), dim3(kThreads),
+                               stream, pl.d_reduce, (long long)k0));
       }
     }
     for (int i : moving) {

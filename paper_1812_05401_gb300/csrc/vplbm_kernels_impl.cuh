@@ -15,14 +15,12 @@ static dim3 node_grid(const StepParams& p) {
 
 template <int COLL>
 static cudaError_t launch_fused_coll(const StepParams& p, cudaStream_t st) {
-  if (p.mode == kModeAAPush) {
-    fused_step_kernel<VPLBM_STORE, COLL, kModeAAPush><<<p.n_tiles, dim3(kLanes, warps_per_block(VPLBM_STORE)), 0, st>>>(p);
-  } else if (p.mode == kModeAALocal) {
-    fused_step_kernel<VPLBM_STORE, COLL, kModeAALocal><<<p.n_tiles, dim3(kLanes, warps_per_block(VPLBM_STORE)), 0, st>>>(p);
-  } else {
-    fused_step_kernel<VPLBM_STORE, COLL, kModeAB><<<p.n_tiles, dim3(kLanes, warps_per_block(VPLBM_STORE)), 0, st>>>(p);
-  }
-  return cudaGetLastError();
+  const dim3 grid(p.n_tiles), blk(kLanes, warps_per_block(VPLBM_STORE));
+  if (p.mode == kModeAAPush)
+    return launch_pdl(fused_step_kernel<VPLBM_STORE, COLL, kModeAAPush>, grid, blk, st, p);
+  if (p.mode == kModeAALocal)
+    return launch_pdl(fused_step_kernel<VPLBM_STORE, COLL, kModeAALocal>, grid, blk, st, p);
+  return launch_pdl(fused_step_kernel<VPLBM_STORE, COLL, kModeAB>, grid, blk, st, p);
 }
 
 cudaError_t VPLBM_FN(launch_fused_)(int coll, const StepParams& p, cudaStream_t st) {
@@ -32,14 +30,12 @@ cudaError_t VPLBM_FN(launch_fused_)(int coll, const StepParams& p, cudaStream_t 
 cudaError_t VPLBM_FN(launch_group_)(const StepParams* d_params, const GroupTile* d_table,
                                     int n_blocks, long long k, int mode, cudaStream_t st) {
   if (n_blocks <= 0) return cudaSuccess;
-  const dim3 blk(kLanes, warps_per_block(VPLBM_STORE));
+  const dim3 grid(n_blocks), blk(kLanes, warps_per_block(VPLBM_STORE));
   if (mode == kModeAAPush)
-    fused_group_kernel<VPLBM_STORE, kModeAAPush><<<n_blocks, blk, 0, st>>>(d_params, d_table, k);
-  else if (mode == kModeAALocal)
-    fused_group_kernel<VPLBM_STORE, kModeAALocal><<<n_blocks, blk, 0, st>>>(d_params, d_table, k);
-  else
-    fused_group_kernel<VPLBM_STORE, kModeAB><<<n_blocks, blk, 0, st>>>(d_params, d_table, k);
-  return cudaGetLastError();
+    return launch_pdl(fused_group_kernel<VPLBM_STORE, kModeAAPush>, grid, blk, st, d_params, d_table, k);
+  if (mode == kModeAALocal)
+    return launch_pdl(fused_group_kernel<VPLBM_STORE, kModeAALocal>, grid, blk, st, d_params, d_table, k);
+  return launch_pdl(fused_group_kernel<VPLBM_STORE, kModeAB>, grid, blk, st, d_params, d_table, k);
 }
 
 cudaError_t VPLBM_FN(launch_moments_)(const StepParams& p, double* rho, double* ux, double* uy,

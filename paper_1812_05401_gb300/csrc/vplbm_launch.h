@@ -7,6 +7,24 @@
 
 namespace vplbm {
 
+// Launch that may start while the previous kernel on the stream still runs:
+// the kernel calls pdl_wait() before its first access to memory that earlier
+// work writes, and pdl_trigger() to let its own successor start. Behind other
+// stream work (a copy, a kernel without a trigger) it is an ordinary launch.
+template <class... Params, class... Args>
+cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, cudaStream_t st, Args&&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 #define VPLBM_DECLARE_LAUNCHERS(SUFFIX)                                                         \
   cudaError_t launch_fused_##SUFFIX(int coll, const StepParams& p, cudaStream_t st);            \
   cudaError_t launch_group_##SUFFIX(const StepParams* d_params,                                 \

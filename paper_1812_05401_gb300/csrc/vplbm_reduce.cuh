@@ -8,6 +8,12 @@
 
 namespace vplbm {
 
+// Programmatic dependent launch (launch_pdl). pdl_trigger: the next launch's
+// blocks may take free slots from here on. pdl_wait: returns once all earlier
+// work on the stream is complete and its writes are visible.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
