@@ -278,6 +278,15 @@ __device__ __forceinline__ unsigned round_bits(unsigned counter, unsigned key) {
 
 
 
+// Explicitly rounded operations. The collision is written with them so that
+// no instance of it depends on which products the compiler contracts: a node
+// has the same bits in every kernel (single, in-place, grouped, paired steps)
+// that computes it.
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // Convective outlet (Section 3.3, after Yang): the ghost column x = nx of
 // direction as (3, 6 or 7), row ys, advanced by the implicit upwind step of
 // dg/dt + U_c dg/dx = 0 from the last column's f*(t):
@@ -291,7 +300,7 @@ __device__ __forceinline__ typename S::T outlet_ghost(const StepParams& p,
   const Consts<T>& c = consts<T>(p);
   const long long gi = (long long)(as == 3 ? 0 : (as == 6 ? 1 : 2)) * p.ny + ys;
   const T f_last = load_h<S>(p, src + (long long)as * p.plane + (long long)ys * p.pitch + (p.nx - 1), as);
-  const T g = (static_cast<const T*>(p.ghost_src)[gi] + c.u_conv * f_last) * c.conv_inv;
+  const T g = mul(mad(c.u_conv, f_last, static_cast<const T*>(p.ghost_src)[gi]), c.conv_inv);
   if (write) static_cast<T*>(p.ghost_dst)[gi] = g;
   return g;
 }
@@ -311,7 +320,7 @@ __device__ __forceinline__ typename S::T outlet_ghost_aa(const StepParams& p, in
     return ESP ? S::in_e(ze, as) : S::in(ze, as, sref<S>(p, as));
   const T f_last = S::in(ze, as, sref<S>(p, as));
   const Consts<T>& c = consts<T>(p);
-  const T g = (static_cast<const T*>(p.ghost_src)[gi] + c.u_conv * f_last) * c.conv_inv;
+  const T g = mul(mad(c.u_conv, f_last, static_cast<const T*>(p.ghost_src)[gi]), c.conv_inv);
   if (write && p.ghost_dst) static_cast<T*>(p.ghost_dst)[gi] = g;
   return ESP ? g - sref<S>(p, as) : g;
 }
@@ -402,8 +411,8 @@ __device__ __forceinline__ void solid_velocity(const StepParams& p, uint8_t m, i
     const T* b = consts<T>(p).body[m - 1];
     const T dx = T(x) - b[0];
     const T dy = T(y) - b[1];
-    usx = b[2] - b[4] * dy;
-    usy = b[3] + b[4] * dx;
+    usx = mad(-b[4], dy, b[2]);
+    usy = mad(b[4], dx, b[3]);
   }
   // any other label (only a caller-written mask can hold one) is solid at rest
 }
@@ -425,11 +434,16 @@ __device__ __forceinline__ T pair_d(const Consts<T>& c, T ha, T hb, int k) {
     return ha - hb;
 }
 
-// FREE: a fluid node (m = 0) without body force (g = 0), for which Eqs. 17
-// and 18 reduce to f_pen = 0 and u = j / rho; the same values as the general
-// form, which would compute them through zero terms.
+// Forms of a node's step. kGeneral: any node. A fluid node (m = 0) without
+// body force (g = 0), for which Eqs. 17 and 18 reduce to f_pen = 0 and
+// u = j / rho, needs half the operations: kFluid gives the general form's
+// bits, which computes the same values through zero terms; kFree rounds the
+// collision's last products in another order. Which of the two a node takes
+// depends on its place alone (free_form), not on the kernel.
 // REF: h holds the elements e = h - h_ref of a 16-bit store.
-template <class T, bool FREE = false, bool REF = false>
+enum { kGeneral = 0, kFluid = 1, kFree = 2 };
+
+template <class T, int FORM = kGeneral, bool REF = false>
 __device__ __forceinline__ Macro<T> macros(const StepParams& p, const T h[9], uint8_t m, int x,
                                            int y) {
   Macro<T> r;
@@ -444,10 +458,10 @@ __device__ __forceinline__ Macro<T> macros(const StepParams& p, const T h[9], ui
   r.rho = T(1) + r.drho;
   const T jx = d13 + (d57 - d68);
   const T jy = d24 + (d57 + d68);
-  if constexpr (FREE) {
+  if constexpr (FORM != kGeneral) {
     const T inv = recip(r.rho);
-    r.ux = jx * inv;
-    r.uy = jy * inv;
+    r.ux = mul(jx, inv);
+    r.uy = mul(jy, inv);
     r.fpx = r.fpy = r.Fx = r.Fy = T(0);
     return r;
   }
@@ -458,15 +472,16 @@ __device__ __forceinline__ Macro<T> macros(const StepParams& p, const T h[9], ui
     solid_velocity<T>(p, m, x, y, usx, usy);
   }
   const T gx = c.gx, gy = c.gy;
-  const T dx = jx + T(0.5) * r.rho * gx - r.rho * usx;
-  const T dy = jy + T(0.5) * r.rho * gy - r.rho * usy;
-  const T inv = recip(r.rho * (T(1) + a));
-  r.ux = usx + dx * inv;
-  r.uy = usy + dy * inv;
-  r.fpx = -kap * dx;
-  r.fpy = -kap * dy;
-  r.Fx = r.fpx + r.rho * gx;
-  r.Fy = r.fpy + r.rho * gy;
+  const T half = mul(T(0.5), r.rho);
+  const T dx = mad(-r.rho, usx, mad(half, gx, jx));
+  const T dy = mad(-r.rho, usy, mad(half, gy, jy));
+  const T inv = recip(mul(r.rho, T(1) + a));
+  r.ux = mad(dx, inv, usx);
+  r.uy = mad(dy, inv, usy);
+  r.fpx = mul(-kap, dx);
+  r.fpy = mul(-kap, dy);
+  r.Fx = mad(r.rho, gx, r.fpx);
+  r.Fy = mad(r.rho, gy, r.fpy);
   return r;
 }
 
@@ -490,41 +505,48 @@ __device__ __forceinline__ Macro<T> macros(const StepParams& p, const T h[9], ui
 // e*_a = e_a + P + Q, with d decoded from the elements (pair_d); r is odd in
 // xi, so s, e_0 = h_0 and the rest population's update need no decoding.
 // ---------------------------------------------------------------------------
-template <class T, bool FREE>
-__device__ __forceinline__ void trt_pair(T& ha, T& hb, T s, T d, T xu, T xF, T kw, T aw, T bw,
+// w: the weight of the pair's directions.
+template <class T, int FORM>
+__device__ __forceinline__ void trt_pair(T& ha, T& hb, T s, T d, T xu, T xF, T K, T w, T aw, T bw,
                                          T amw, T bmw, T hsp, T hsm) {
-  // w (s+ heq+ + c+ G+) and w (s- heq- + c- G-); without a force G+- = 0
-  const T rp = FREE ? xu * (aw * xu) + kw : xu * (aw * xu + bw * xF) + kw;
-  const T rm = FREE ? amw * xu : amw * xu + bmw * xF;
-  const T P = rp - hsp * s;
-  const T Q = rm - hsm * d;
+  // P = w (s+ heq+ + c+ G+) - (s+/2) s and Q = w (s- heq- + c- G-) - (s-/2) d;
+  // without a force G+- = 0
+  T P, Q;
+  if constexpr (FORM == kFree) {
+    P = mad(-hsp, s, mad(xu, mul(aw, xu), mul(K, w)));
+    Q = mad(amw, xu, -mul(hsm, d));
+  } else if constexpr (FORM == kFluid) {
+    P = mad(-hsp, s, mad(K, w, mul(xu, mul(aw, xu))));
+    Q = mad(-hsm, d, mul(amw, xu));
+  } else {
+    P = mad(-hsp, s, mad(K, w, mul(xu, mad(aw, xu, mul(bw, xF)))));
+    Q = mad(-hsm, d, mad(amw, xu, mul(bmw, xF)));
+  }
   ha = ha + (P + Q);
   hb = hb + (P - Q);
 }
 
-template <class T, bool FREE = false, bool REF = false>
+template <class T, int FORM = kGeneral, bool REF = false>
 __device__ __forceinline__ void collide_trt(const StepParams& p, T h[9], const Macro<T>& q) {
   const Consts<T>& c = consts<T>(p);
   const T ux = q.ux, uy = q.uy, Fx = q.Fx, Fy = q.Fy, rho = q.rho;
-  const T uu = ux * ux + uy * uy;
-  const T K = FREE ? c.t_sp * (q.drho - T(1.5) * rho * uu)
-                   : c.t_sp * (q.drho - T(1.5) * rho * uu) - c.t_c3p * (ux * Fx + uy * Fy);
-  const T k9 = K * T(1.0 / 9.0), k36 = K * T(1.0 / 36.0);
-  const T a9 = c.t_a[0] * rho, a36 = c.t_a[1] * rho;
-  const T am9 = c.t_am[0] * rho, am36 = c.t_am[1] * rho;
+  const T w9 = T(1.0 / 9.0), w36 = T(1.0 / 36.0);
+  const T uu = mad(ux, ux, mul(uy, uy));
+  const T e = mad(-mul(T(1.5), rho), uu, q.drho);
+  const T K = FORM != kGeneral ? mul(c.t_sp, e) : mad(c.t_sp, e, -mul(c.t_c3p, mad(ux, Fx, mul(uy, Fy))));
+  const T a9 = mul(c.t_a[0], rho), a36 = mul(c.t_a[1], rho);
+  const T am9 = mul(c.t_am[0], rho), am36 = mul(c.t_am[1], rho);
   // the pair sums and differences as macros() formed them
   const T s13 = pair_s<T>(h[1], h[3]), s24 = pair_s<T>(h[2], h[4]);
   const T s57 = pair_s<T>(h[5], h[7]), s68 = pair_s<T>(h[6], h[8]);
   const T d13 = pair_d<T, REF>(c, h[1], h[3], 0), d24 = pair_d<T, REF>(c, h[2], h[4], 1);
   const T d57 = pair_d<T, REF>(c, h[5], h[7], 2), d68 = pair_d<T, REF>(c, h[6], h[8], 3);
-  h[0] = c.t_1msp * h[0] + T(4.0 / 9.0) * K;
-  trt_pair<T, FREE>(h[1], h[3], s13, d13, ux, Fx, k9, a9, c.t_b[0], am9, c.t_bm[0], c.t_hsp,
-                    c.t_hsm);
-  trt_pair<T, FREE>(h[2], h[4], s24, d24, uy, Fy, k9, a9, c.t_b[0], am9, c.t_bm[0], c.t_hsp,
-                    c.t_hsm);
-  trt_pair<T, FREE>(h[5], h[7], s57, d57, ux + uy, Fx + Fy, k36, a36, c.t_b[1], am36, c.t_bm[1],
+  h[0] = mad(T(4.0 / 9.0), K, mul(c.t_1msp, h[0]));
+  trt_pair<T, FORM>(h[1], h[3], s13, d13, ux, Fx, K, w9, a9, c.t_b[0], am9, c.t_bm[0], c.t_hsp, c.t_hsm);
+  trt_pair<T, FORM>(h[2], h[4], s24, d24, uy, Fy, K, w9, a9, c.t_b[0], am9, c.t_bm[0], c.t_hsp, c.t_hsm);
+  trt_pair<T, FORM>(h[5], h[7], s57, d57, ux + uy, Fx + Fy, K, w36, a36, c.t_b[1], am36, c.t_bm[1],
                     c.t_hsp, c.t_hsm);
-  trt_pair<T, FREE>(h[6], h[8], s68, d68, uy - ux, Fy - Fx, k36, a36, c.t_b[1], am36, c.t_bm[1],
+  trt_pair<T, FORM>(h[6], h[8], s68, d68, uy - ux, Fy - Fx, K, w36, a36, c.t_b[1], am36, c.t_bm[1],
                     c.t_hsp, c.t_hsm);
 }
 
@@ -598,20 +620,22 @@ __device__ __forceinline__ void collide_mrt(const StepParams& p, T h[9], const M
 // Every direction is pulled with one N-element vector load per lane: a
 // direction with xi_x = +1 takes its first node's value from the lane to the
 // left (warp shuffle), one with xi_x = -1 its last node's value from the lane
-// to the right, and only the edge lanes 0 and 31 load that one value
-// themselves. Interior tiles (no boundary within one node) do nothing else.
-// Tiles touching a boundary (GEN) also remap: the source row of each direction
-// (periodic wrap or free-slip mirror, uniform across the warp), the edge
-// lanes' single values (periodic wrap, inlet ghost, outlet copy), and the value
-// entering the domain's last column; lanes past the last column load and
-// store nothing. The arithmetic per node is the same on both paths.
+// to the right. The values from beside the tile come with one more load, one
+// value per lane (EdgeLane), and are handed to the edge lanes by shuffles.
+// Interior tiles (no boundary within one node) do nothing else. Tiles touching
+// a boundary (GEN) also remap: the source row of each direction (periodic wrap
+// or free-slip mirror, uniform across the warp), the values from beside the
+// tile (periodic wrap, inlet ghost, outlet copy), and those entering the
+// domain's last column; lanes past the last column load and store nothing.
 // ---------------------------------------------------------------------------
+// The value of direction as from (xs, ys), through the x boundary rules (the
+// caller has applied the y rules to as and ys).
 // AA: the push step reads f*_as(xs, ys) from the opposite slot of the source
 // node (where the local step put it).
-// ESP: the value as an element of direction A (offset minus the reference),
-// as the fused step works on them; the reference is even in xi_y, so the
-// mirrored source as of a free-slip wall has A's reference.
-template <class S, int A, bool AA = false, bool ESP = false>
+// ESP: the value as an element (offset minus the reference), as the fused step
+// works on them; the reference is even in xi_y, so the mirrored source as of a
+// free-slip wall has the pulled direction's reference.
+template <class S, bool AA = false, bool ESP = false>
 __device__ __forceinline__ typename S::T edge_pull(const StepParams& p, const typename S::E* src,
                                                    int as, int ys, int xs) {
   using T = typename S::T;
@@ -620,16 +644,14 @@ __device__ __forceinline__ typename S::T edge_pull(const StepParams& p, const ty
       xs %= p.nx;
       if (xs < 0) xs += p.nx;
     } else if (xs < 0) {  // inlet ghost column at f_eq(1, u_in)
-      const Consts<T>& c = consts<T>(p);
-      const T h = as == A ? c.heq_in[A] : c.heq_in[mirror_y(A)];
-      return ESP ? h - sref<S>(p, A) : h;
+      const T h = consts<T>(p).heq_in[as];
+      return ESP ? h - sref<S>(p, as) : h;
     } else if (AA) {
       return outlet_ghost_aa<S, ESP>(p, as, ys, xs == p.nx);
     } else if (p.bc_x == kBcInletConvective) {
-      // xs == nx: the last column's own pull (the entry's one reader); beyond
-      // it, the unused edge value of a lane past the last column
+      // xs == nx: the last column's own pull (the entry's one reader)
       const T g = outlet_ghost<S>(p, src, as, ys, xs == p.nx);
-      return ESP ? g - sref<S>(p, A) : g;
+      return ESP ? g - sref<S>(p, as) : g;
     } else {  // zero-gradient outlet ghost column
       xs = p.nx - 1;
     }
@@ -638,58 +660,129 @@ __device__ __forceinline__ typename S::T edge_pull(const StepParams& p, const ty
   return ESP ? S::in_e(e, as) : S::in(e, as, sref<S>(p, as));
 }
 
-template <class S, int N, int A, bool GEN, bool AA = false>
-__device__ __forceinline__ void pull_dir_vec(const StepParams& p, const typename S::E* src, int xb,
-                                             int y, int lane, bool lane_active,
-                                             typename S::T (&h)[N][9]) {
+// Place of a direction with xi_x != 0 among the three of its side (1, 5, 8 and
+// 3, 6, 7: xi_y = 0, 1, -1).
+__device__ __forceinline__ constexpr int side_slot(int a) {
+  return a == 1 || a == 3 ? 0 : (a == 5 || a == 6 ? 1 : 2);
+}
+
+// The values that enter a row of a tile from beside it, one per lane (so that
+// one load covers them all): lanes 0..2 take directions 1, 5, 8 from x0 - 1,
+// lanes 3..5 directions 3, 6, 7 from x0 + TX, and in the tile of the domain's
+// last column (GEN) lanes 6..8 directions 3, 6, 7 from beyond that column. As
+// one load per direction by the edge lane alone they were six more loads per
+// row of an interior tile, and in boundary tiles nine instances of the
+// boundary rules, run one after the other. With it, per step: 1001 x 701 BF16
+// 19.7 -> 14.1 us, 4096 x 1024 FP32 58.3 -> 51.7 and FP16 43.8 -> 36.7 us,
+// 16384 x 4096 FP16 0.483 -> 0.454 ms, 32 mixed solves 344 -> 284 us (with
+// the branch-free rows of collide_row for FP32). The interior tiles' source is
+// kept as one pointer: worked out anew in each row, the 16384 x 4096 FP16 step
+// took 0.51 ms; three loads by lanes 0 and 31 in place of one and six shuffles
+// likewise.
+template <class S, int TX, bool GEN, bool AA = false>
+struct EdgeLane {
   using T = typename S::T;
   using E = typename S::E;
-  int as = A;
-  int ys = y - cy(A);
-  if (GEN && (ys < 0 || ys >= p.ny)) {
-    if (p.bc_y == kBcPeriodic) {
-      ys = ys < 0 ? ys + p.ny : ys - p.ny;
-    } else {  // free slip: the mirror of the population that left this row
-      as = mirror_y(A);
-      ys = y;
+  const E* at;  // interior tiles: the lane's source in row 0 (null: none)
+  __device__ __forceinline__ EdgeLane(const StepParams& p, const E* src, int x0, int lane) {
+    if constexpr (!GEN) {
+      const int m = lane % 3;
+      const bool left = lane < 3;
+      const int a = m == 0 ? (left ? 1 : 3) : (m == 1 ? (left ? 5 : 6) : (left ? 8 : 7));
+      const int dy = m == 0 ? 0 : (m == 1 ? -1 : 1);
+      at = lane < 6 ? src + (long long)(AA ? opposite(a) : a) * p.plane + dy * p.pitch + (left ? x0 - 1 : x0 + TX)
+                    : nullptr;
     }
   }
-  const E* row = src + (long long)(AA ? opposite(as) : as) * p.plane + (long long)ys * p.pitch;
-  T v[N];
-  if (!GEN || lane_active) {
-    S::load_h(row + xb, v, as);
-  } else {
-#pragma unroll
-    for (int k = 0; k < N; ++k) v[k] = T(0);
-  }
-  if (cx(A) == 0) {
-#pragma unroll
-    for (int k = 0; k < N; ++k) h[k][A] = v[k];
-  } else if (cx(A) == 1) {  // node k pulls from x - 1
-    T left = __shfl_up_sync(0xffffffffu, v[N - 1], 1);
-    // the edge lanes' extra value: through the x boundary rules only where
-    // it lies outside the grid (the source row already carries the y rules)
-    if (lane == 0)
-      left = GEN && xb - 1 < 0 ? edge_pull<S, A, AA, true>(p, src, as, ys, xb - 1)
-                               : S::in_e(row[xb - 1], as);
-    h[0][A] = left;
-#pragma unroll
-    for (int k = 1; k < N; ++k) h[k][A] = v[k - 1];
-  } else {  // node k pulls from x + 1
-    T right = __shfl_down_sync(0xffffffffu, v[0], 1);
-    if (lane == kLanes - 1)
-      right = GEN && xb + N >= p.nx ? edge_pull<S, A, AA, true>(p, src, as, ys, xb + N)
-                                    : S::in_e(row[xb + N], as);
-#pragma unroll
-    for (int k = 0; k < N - 1; ++k) h[k][A] = v[k + 1];
-    h[N - 1][A] = right;
-    if (GEN && xb <= p.nx - 1 && xb + N > p.nx - 1) {
-      // the domain's last column pulls from beyond it, through the x boundary
-#pragma unroll
-      for (int k = 0; k < N; ++k)
-        if (xb + k == p.nx - 1) h[k][A] = edge_pull<S, A, AA, true>(p, src, as, ys, p.nx);
+  __device__ __forceinline__ T value(const StepParams& p, const E* src, int x0, int y, int lane) const {
+    if constexpr (!GEN) {
+      // FP64 weights: 1/9 for xi_y = 0, 1/36 for the others
+      return at ? S::in_e(at[(long long)y * p.pitch], lane % 3 == 0 ? 1 : 5) : T(0);
+    } else {
+      const bool last = x0 + TX >= p.nx;
+      if (lane >= 9 || (last ? lane >= 3 && lane < 6 : lane >= 6)) return T(0);
+      const int m = lane % 3;
+      const bool left = lane < 3;
+      int as = m == 0 ? (left ? 1 : 3) : (m == 1 ? (left ? 5 : 6) : (left ? 8 : 7));
+      int ys = y - (m == 0 ? 0 : (m == 1 ? 1 : -1));
+      if (ys < 0 || ys >= p.ny) {
+        if (p.bc_y == kBcPeriodic) {
+          ys = ys < 0 ? ys + p.ny : ys - p.ny;
+        } else {
+          as = m == 1 ? (left ? 8 : 7) : (left ? 5 : 6);
+          ys = y;
+        }
+      }
+      return edge_pull<S, AA, true>(p, src, as, ys, left ? x0 - 1 : (last ? p.nx : x0 + TX));
     }
   }
+};
+
+// Node k's pulled value from the loaded vectors: its own place's for xi_x = 0,
+// the left or right neighbour's for xi_x = +-1 (from the neighbouring lane, or
+// from edge, the values of EdgeLane, at the row's ends).
+template <class S, int N, bool GEN>
+__device__ __forceinline__ void shift_row(int nx, int x0, int lane, const typename S::T (&v)[9][N],
+                                          typename S::T edge, typename S::T (&h)[N][9]) {
+  using T = typename S::T;
+#pragma unroll
+  for (int a = 0; a < 9; ++a) {
+    if (cx(a) == 0) {
+#pragma unroll
+      for (int k = 0; k < N; ++k) h[k][a] = v[a][k];
+    } else if (cx(a) == 1) {
+      const T left = __shfl_up_sync(0xffffffffu, v[a][N - 1], 1);
+      const T e = __shfl_sync(0xffffffffu, edge, side_slot(a));
+      h[0][a] = lane == 0 ? e : left;
+#pragma unroll
+      for (int k = 1; k < N; ++k) h[k][a] = v[a][k - 1];
+    } else {
+      const T right = __shfl_down_sync(0xffffffffu, v[a][0], 1);
+      const T e = __shfl_sync(0xffffffffu, edge, 3 + side_slot(a));
+#pragma unroll
+      for (int k = 0; k < N - 1; ++k) h[k][a] = v[a][k + 1];
+      h[N - 1][a] = lane == kLanes - 1 ? e : right;
+      if (GEN && x0 + kLanes * N >= nx) {  // the domain's last column
+        const T beyond = __shfl_sync(0xffffffffu, edge, 6 + side_slot(a));
+        const int at = nx - 1 - x0 - lane * N;
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+          if (k == at) h[k][a] = beyond;
+      }
+    }
+  }
+}
+
+// The pulled populations of a lane's N nodes xb .. xb + N - 1 of row y.
+template <class S, int N, bool GEN, bool AA = false>
+__device__ __forceinline__ void pull_row(const StepParams& p, const typename S::E* src,
+                                         const EdgeLane<S, kLanes * N, GEN, AA>& el, int x0, int y, int lane,
+                                         bool lane_active, typename S::T (&h)[N][9]) {
+  using T = typename S::T;
+  using E = typename S::E;
+  const T edge = el.value(p, src, x0, y, lane);
+  const int xb = x0 + lane * N;
+  T v[9][N];
+#pragma unroll
+  for (int a = 0; a < 9; ++a) {
+    int as = a, ys = y - cy(a);
+    if (GEN && (ys < 0 || ys >= p.ny)) {
+      if (p.bc_y == kBcPeriodic) {
+        ys = ys < 0 ? ys + p.ny : ys - p.ny;
+      } else {  // free slip: the mirror of the population that left this row
+        as = mirror_y(a);
+        ys = y;
+      }
+    }
+    const E* row = src + (long long)(AA ? opposite(as) : as) * p.plane + (long long)ys * p.pitch;
+    if (!GEN || lane_active) {
+      S::load_h(row + xb, v[a], a);
+    } else {
+#pragma unroll
+      for (int k = 0; k < N; ++k) v[a][k] = T(0);
+    }
+  }
+  shift_row<S, N, GEN>(p.nx, x0, lane, v, edge, h);
 }
 
 // ---------------------------------------------------------------------------
@@ -862,7 +955,7 @@ __device__ __forceinline__ void aa_local_boundary(const StepParams& p, typename 
     } else if (p.bc_x == kBcInletConvective) {
       const long long gi = (long long)(as == 3 ? 0 : (as == 6 ? 1 : 2)) * p.ny + ys;
       const T f_last = ESP ? h[a] + sref<S>(p, a) : h[a];
-      const T g = (static_cast<const T*>(p.ghost_src)[gi] + c.u_conv * f_last) * c.conv_inv;
+      const T g = mul(mad(c.u_conv, f_last, static_cast<const T*>(p.ghost_src)[gi]), c.conv_inv);
       if (write) static_cast<T*>(p.ghost_dst)[gi] = g;
       h[a] = ESP ? g - sref<S>(p, a) : g;
     }
@@ -883,6 +976,183 @@ __device__ __forceinline__ typename S::E fstar_e(const StepParams& p, const type
   return static_cast<const typename S::E*>(p.lost)[lost_index(p, a, y, x + cx(a) < 0)];
 }
 
+// What a thread adds up for a step's record over the rows it collides: sum of
+// drho, and the force on its solid nodes (<= 16, arithmetic type).
+template <class T>
+struct RowSums {
+  T dm = T(0), fx = T(0), fy = T(0);
+  bool solid = false;
+};
+
+// The N mask bytes of a lane's nodes, byte k for node k (kept in one register:
+// the collision's registers are the kernel's tightest budget).
+template <int N>
+__device__ __forceinline__ unsigned mask_word(const uint8_t* m) {
+  return N == 4 ? *reinterpret_cast<const unsigned*>(m) : unsigned(*reinterpret_cast<const unsigned short*>(m));
+}
+
+// Whether the tile at column tx and row ty of tiles touches no boundary: none
+// of its nodes pulls from outside the grid.
+template <int STORE>
+__device__ __forceinline__ bool interior_tile(const StepParams& p, int tx, int ty) {
+  const int x0 = tx * tile_x(STORE), y0 = ty * p.tile_y;
+  return x0 >= 1 && x0 + tile_x(STORE) <= p.nx - 1 && y0 >= 1 && y0 + p.tile_y <= p.ny - 1;
+}
+
+// Whether fluid nodes of a tile take the force-free form of the step.
+template <int STORE>
+__device__ __forceinline__ bool free_form(const StepParams& p, int tx, int ty) {
+  return p.force_free && interior_tile<STORE>(p, tx, ty);
+}
+
+// Storages whose rows of fluid nodes are collided without branches: FP32, and
+// FP64 (1024 x 256 step 82.0 -> 79.0 us). The 16-bit kernels, at 64 registers,
+// lose by it (4096 x 1024 FP16 batch of 50 steps 2.00 -> 2.03 ms).
+__host__ __device__ constexpr bool straight_rows(int storage) { return storage == kF32 || storage == kF64; }
+
+// Collide one row's N pulled nodes of a lane whose first node lies in the
+// domain. free: fluid nodes take the force-free form (free_form of their tile).
+template <int STORE, int COLL, bool GEN, int N>
+__device__ __forceinline__ void collide_row(const StepParams& p, typename Store<STORE>::T (&h)[N][9],
+                                            unsigned mw, int xb, int y, bool free,
+                                            RowSums<typename Store<STORE>::T>& acc) {
+  using S = Store<STORE>;
+  using T = typename S::T;
+  constexpr bool REF = S::kSixteen;  // h holds elements e = h - h_ref
+  auto finish_node = [&](const Macro<T>& q, uint8_t m) {
+    // a NaN or infinite population makes rho NaN, infinite or non-positive
+    if (!(q.rho > T(0) && q.rho < T(1e30))) atomicOr(p.flag, 1);
+    acc.dm += q.drho;
+    if (m) {
+      acc.solid = true;
+      acc.fx -= q.fpx;
+      acc.fy -= q.fpy;
+    }
+  };
+  // A row of fluid nodes only, without body force (a warp's usual row): the
+  // lane's nodes one beside the other without a branch between them, so that
+  // their dependent chains overlap. Interior tiles take kFree there and
+  // boundary tiles kFluid.
+  if (COLL == kTrt && straight_rows(STORE) && p.force_free && free != GEN &&
+      (!GEN || xb + (kLanes - int(threadIdx.x)) * N <= p.nx) && !__any_sync(0xffffffffu, mw != 0)) {
+    constexpr int FORM = GEN ? kFluid : kFree;
+    bool sound = true;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const Macro<T> q = macros<T, FORM, REF>(p, h[k], 0, xb + k, y);
+      collide_trt<T, FORM, REF>(p, h[k], q);
+      sound = sound && q.rho > T(0) && q.rho < T(1e30);
+      acc.dm += q.drho;
+    }
+    if (!sound) atomicOr(p.flag, 1);
+    return;
+  }
+  auto node = [&](T(&hk)[9], int x, uint8_t m) {
+    if (GEN && x >= p.nx) return;  // past the last column: padding, stored as pulled
+    if (COLL == kTrt && free && m == 0) {
+      // a fluid node without body force
+      const Macro<T> q = macros<T, kFree, REF>(p, hk, 0, x, y);
+      collide_trt<T, kFree, REF>(p, hk, q);
+      finish_node(q, 0);
+    } else if (COLL == kTrt) {
+      const Macro<T> q = macros<T, kGeneral, REF>(p, hk, m, x, y);
+      collide_trt<T, kGeneral, REF>(p, hk, q);
+      finish_node(q, m);
+    } else {
+      // the moment-space form works on offsets
+      if constexpr (REF) {
+#pragma unroll
+        for (int a = 0; a < 9; ++a) hk[a] = hk[a] + sref<S>(p, a);
+      }
+      const Macro<T> q = macros<T>(p, hk, m, x, y);
+      collide_mrt<T>(p, hk, q);
+      finish_node(q, m);
+      if constexpr (REF) {
+#pragma unroll
+        for (int a = 0; a < 9; ++a) hk[a] = hk[a] - sref<S>(p, a);
+      }
+    }
+  };
+#pragma unroll
+  for (int k = 0; k < N; ++k) node(h[k], xb + k, uint8_t(mw >> (8 * k)));
+}
+
+// The rounding word of each of a lane's node pairs (16-bit stores): pairs
+// (xb, xb + 1), (xb + 2, xb + 3) are numbered row by row.
+template <int NW>
+__device__ __forceinline__ void round_words(const StepParams& p, int xb, int y, unsigned key, bool sr,
+                                            unsigned (&nb)[NW]) {
+#pragma unroll
+  for (int j = 0; j < NW; ++j)
+    nb[j] = sr ? round_bits(unsigned((long long)y * ((p.nx + 1) >> 1) + (xb >> 1) + j), key) : 0u;
+}
+
+// The tile's share of the records of K steps (reduce_kernel adds the tiles):
+// the force on the solid nodes, summed per thread in the arithmetic type (each
+// thread holds at most 16 nodes) and in FP64 from the thread up; the total
+// density, in the arithmetic type within the block and FP64 from the tile up.
+// Warps and blocks without solid nodes skip the FP64 work (on GB300 FP64 runs
+// at a small fraction of the FP32 rate).
+template <int STORE, int K>
+__device__ __forceinline__ void tile_records(const StepParams& p, int tile, int x0, int y0,
+                                             const RowSums<typename Store<STORE>::T> (&acc)[K],
+                                             double* const (&partials)[K]) {
+  using T = typename Store<STORE>::T;
+  constexpr int W = warps_per_block(STORE);
+  constexpr int TX = tile_x(STORE);
+  __shared__ double sm[K][W][2];
+  __shared__ T smass[K][W];
+  const int lane = threadIdx.x, warp = threadIdx.y;
+  const int tid = lane + warp * kLanes;
+  bool block_solid[K];
+#pragma unroll
+  for (int i = 0; i < K; ++i) {
+    const bool warp_solid = __any_sync(0xffffffffu, acc[i].solid);
+    T dm = acc[i].dm;
+    double bfx = 0.0, bfy = 0.0;
+    if (warp_solid) {
+      bfx = double(acc[i].fx);
+      bfy = double(acc[i].fy);
+    }
+    if (p.reduce_mass) dm = warp_sum(dm);
+    if (warp_solid) {
+      bfx = warp_sum(bfx);
+      bfy = warp_sum(bfy);
+    }
+    if (lane == 0) {
+      smass[i][warp] = dm;
+      sm[i][warp][0] = bfx;
+      sm[i][warp][1] = bfy;
+    }
+    block_solid[i] = __syncthreads_or(acc[i].solid);
+  }
+  if (tid == 0) {
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      double ts[3] = {0.0, 0.0, 0.0};
+      T msum = T(0);
+#pragma unroll
+      for (int w = 0; w < W; ++w) msum += smass[i][w];
+      if (block_solid[i]) {
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+          ts[0] += sm[i][w][0];
+          ts[1] += sm[i][w][1];
+        }
+      }
+      if (p.reduce_mass) {
+        // sum rho = active nodes + sum drho
+        const int nact = min(TX, p.nx - x0) * min(p.tile_y, p.ny - y0);
+        ts[2] = double(nact) + double(msum);
+      }
+      double* out = partials[i] + 3ll * tile;
+      out[0] = ts[0];
+      out[1] = ts[1];
+      out[2] = ts[2];
+    }
+  }
+}
+
 // MODE: kModeAB (pull from p.src, store to p.dst), or one of the two in-place
 // AA steps on the one buffer p.dst (== p.src).
 template <int STORE, int COLL, int MODE = kModeAB>
@@ -894,15 +1164,13 @@ __device__ __forceinline__ void step_tile(const StepParams& p, int tile, long lo
   constexpr int N = npt(STORE);
   constexpr int TX = kLanes * N;
   constexpr int W = warps_per_block(STORE);
-  __shared__ double sm[W][3];
-  __shared__ T smass[W];
 
   const int lane = threadIdx.x, warp = threadIdx.y;
   const int tx = tile % p.tiles_x;
   const int ty = tile / p.tiles_x;
   const int x0 = tx * TX, y0 = ty * p.tile_y;
   const int xb = x0 + lane * N;
-  const bool interior = x0 >= 1 && x0 + TX <= p.nx - 1 && y0 >= 1 && y0 + p.tile_y <= p.ny - 1;
+  const bool interior = interior_tile<STORE>(p, tx, ty);
   // Plain pointers and loads: the previous step's stores may complete while
   // this kernel's blocks already wait (pdl_wait), so a load must not be taken
   // for one of memory that stays unchanged for the whole kernel.
@@ -910,67 +1178,19 @@ __device__ __forceinline__ void step_tile(const StepParams& p, int tile, long lo
   E* dst = static_cast<E*>(p.dst);
   E* buf = static_cast<E*>(p.dst);  // the in-place modes' one buffer
 
-  T dm = T(0);           // sum of drho over this thread's nodes
-  T tfx = T(0), tfy = T(0);  // force on this thread's solid nodes (<= 16, arithmetic type)
-  bool any_solid = false;
+  RowSums<T> acc[1];
   const unsigned key = round_bits(unsigned(t), p.round_key);
-
-  auto finish_node = [&](const Macro<T>& q, uint8_t m) {
-    // a NaN or infinite population makes rho NaN, infinite or non-positive
-    if (!(q.rho > T(0) && q.rho < T(1e30))) atomicOr(p.flag, 1);
-    dm += q.drho;
-    if (m) {
-      any_solid = true;
-      tfx -= q.fpx;
-      tfy -= q.fpy;
-    }
-  };
 
   // Collide and store one row of pulled populations (lane_active: the lane's
   // first node lies in the domain).
   auto process_row = [&](int y, auto& h, auto gen) {
     constexpr bool GEN = decltype(gen)::value;
     const long long i = (long long)y * p.pitch + xb;
-    // the N mask bytes of this lane's nodes, byte k for node k (kept in one
-    // register: the collision's registers are the kernel's tightest budget)
-    const unsigned mw = N == 4 ? *reinterpret_cast<const unsigned*>(p.mask + i)
-                               : unsigned(*reinterpret_cast<const unsigned short*>(p.mask + i));
-    auto mk = [&](int k) -> uint8_t { return uint8_t(mw >> (8 * k)); };
+    const unsigned mw = mask_word<N>(p.mask + i);
     const bool sr = S::kSixteen && p.stochastic;
-    constexpr bool REF = S::kSixteen;  // h holds elements e = h - h_ref
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-      if (GEN && xb + k >= p.nx) continue;  // past the last column: padding, stored as pulled
-      if (COLL == kTrt && !GEN && p.force_free && mk(k) == 0) {
-        // a fluid node without body force: the force-free form of the step
-        const Macro<T> q = macros<T, true, REF>(p, h[k], 0, xb + k, y);
-        collide_trt<T, true, REF>(p, h[k], q);
-        finish_node(q, 0);
-      } else if (COLL == kTrt) {
-        const Macro<T> q = macros<T, false, REF>(p, h[k], mk(k), xb + k, y);
-        collide_trt<T, false, REF>(p, h[k], q);
-        finish_node(q, mk(k));
-      } else {
-        // the moment-space form works on offsets
-        if constexpr (REF) {
-#pragma unroll
-          for (int a = 0; a < 9; ++a) h[k][a] = h[k][a] + sref<S>(p, a);
-        }
-        const Macro<T> q = macros<T>(p, h[k], mk(k), xb + k, y);
-        collide_mrt<T>(p, h[k], q);
-        finish_node(q, mk(k));
-        if constexpr (REF) {
-#pragma unroll
-          for (int a = 0; a < 9; ++a) h[k][a] = h[k][a] - sref<S>(p, a);
-        }
-      }
-    }
-    // the rounding word of each of the lane's node pairs (16-bit stores):
-    // pairs (xb, xb + 1), (xb + 2, xb + 3) are numbered row by row
+    collide_row<STORE, COLL, GEN>(p, h, mw, xb, y, !GEN && p.force_free, acc[0]);
     unsigned nb[(N + 1) / 2];
-#pragma unroll
-    for (int j = 0; j < (N + 1) / 2; ++j)
-      nb[j] = sr ? round_bits(unsigned((long long)y * ((p.nx + 1) >> 1) + (xb >> 1) + j), key) : 0u;
+    round_words(p, xb, y, key, sr, nb);
     if constexpr (MODE == kModeAB) {
 #pragma unroll
       for (int a = 0; a < 9; ++a) {
@@ -1028,7 +1248,9 @@ __device__ __forceinline__ void step_tile(const StepParams& p, int tile, long lo
     }
   };
 
-  auto do_row = [&](int y, auto gen) {
+  constexpr bool AA = MODE == kModeAAPush;
+  const E* from = AA ? buf : src;
+  auto do_row = [&](int y, auto gen, const auto& el) {
     constexpr bool GEN = decltype(gen)::value;
     const bool lane_active = !GEN || xb < p.nx;
     T h[N][9];
@@ -1048,82 +1270,29 @@ __device__ __forceinline__ void step_tile(const StepParams& p, int tile, long lo
           if (xb + k < p.nx) aa_local_boundary<S, true>(p, h[k], xb + k, y, true);
       }
     } else {
-      constexpr bool AA = MODE == kModeAAPush;
-      const E* from = AA ? buf : src;
-      pull_dir_vec<S, N, 0, GEN, AA>(p, from, xb, y, lane, lane_active, h);
-      pull_dir_vec<S, N, 1, GEN, AA>(p, from, xb, y, lane, lane_active, h);
-      pull_dir_vec<S, N, 2, GEN, AA>(p, from, xb, y, lane, lane_active, h);
-      pull_dir_vec<S, N, 3, GEN, AA>(p, from, xb, y, lane, lane_active, h);
-      pull_dir_vec<S, N, 4, GEN, AA>(p, from, xb, y, lane, lane_active, h);
-      pull_dir_vec<S, N, 5, GEN, AA>(p, from, xb, y, lane, lane_active, h);
-      pull_dir_vec<S, N, 6, GEN, AA>(p, from, xb, y, lane, lane_active, h);
-      pull_dir_vec<S, N, 7, GEN, AA>(p, from, xb, y, lane, lane_active, h);
-      pull_dir_vec<S, N, 8, GEN, AA>(p, from, xb, y, lane, lane_active, h);
+      pull_row<S, N, GEN, AA>(p, from, el, x0, y, lane, lane_active, h);
       if (!lane_active) return;
     }
     process_row(y, h, gen);
   };
 
   if (interior) {
+    const EdgeLane<S, TX, false, AA> el(p, from, x0, lane);
 #pragma unroll 1
-    for (int r = 0; r < p.rows_per_warp; ++r) do_row(y0 + warp + r * W, std::false_type());
+    for (int r = 0; r < p.rows_per_warp; ++r) do_row(y0 + warp + r * W, std::false_type(), el);
   } else {
+    const EdgeLane<S, TX, true, AA> el(p, from, x0, lane);
 #pragma unroll 1
     for (int r = 0; r < p.rows_per_warp; ++r) {
       const int y = y0 + warp + r * W;
       if (y >= p.ny) break;  // warp-uniform: a warp is one row
-      do_row(y, std::true_type());
+      do_row(y, std::true_type(), el);
     }
   }
 
   pdl_trigger();
-
-  // Per-step record: the force on the solid nodes, summed per thread in the
-  // arithmetic type (each thread holds at most 16 nodes) and in FP64 from the
-  // thread up; the total density, in the arithmetic type within the block and
-  // FP64 from the tile up. Warps and blocks without solid nodes skip the FP64
-  // work (on GB300 FP64 runs at a small fraction of the FP32 rate).
-  const int tid = lane + warp * kLanes;
-  const bool warp_solid = __any_sync(0xffffffffu, any_solid);
-  double bfx = 0.0, bfy = 0.0;
-  if (warp_solid) {
-    bfx = double(tfx);
-    bfy = double(tfy);
-  }
-  if (p.reduce_mass) dm = warp_sum(dm);
-  if (warp_solid) {
-    bfx = warp_sum(bfx);
-    bfy = warp_sum(bfy);
-  }
-  if (lane == 0) {
-    smass[warp] = dm;
-    sm[warp][0] = bfx;
-    sm[warp][1] = bfy;
-  }
-  const int block_solid = __syncthreads_or(any_solid);
-  if (tid == 0) {
-    double ts[3] = {0.0, 0.0, 0.0};
-    T msum = T(0);
-#pragma unroll
-    for (int w = 0; w < W; ++w) msum += smass[w];
-    if (block_solid) {
-#pragma unroll
-      for (int w = 0; w < W; ++w) {
-        ts[0] += sm[w][0];
-        ts[1] += sm[w][1];
-      }
-    }
-    if (p.reduce_mass) {
-      // sum rho = active nodes + sum drho
-      const int nact = min(TX, p.nx - x0) * min(p.tile_y, p.ny - y0);
-      ts[2] = double(nact) + double(msum);
-    }
-    // the tile's share of the step's record; reduce_kernel adds the tiles
-    double* out = partials + 3ll * tile;
-    out[0] = ts[0];
-    out[1] = ts[1];
-    out[2] = ts[2];
-  }
+  double* const parts[1] = {partials};
+  tile_records<STORE>(p, tile, x0, y0, acc, parts);
 }
 
 // Consecutive steps are launched dependently (launch_pdl): once every block has
@@ -1192,7 +1361,7 @@ __device__ __forceinline__ typename S::T pull_aa(const StepParams& p, const type
       ys = y;
     }
   }
-  return edge_pull<S, A, true>(p, buf, as, ys, x - cx(A));
+  return edge_pull<S, true>(p, buf, as, ys, x - cx(A));
 }
 template <class S>
 __device__ __forceinline__ void pull_node_any(const StepParams& p, int x, int y, typename S::T h[9]) {
