@@ -206,7 +206,7 @@ struct vplbm_solver {
   int cur = 0;  // buffer holding f*(t)
   uint8_t* mask = nullptr;
   void* us = nullptr;
-  double* partials = nullptr;    // [kWindow][n_tiles][3]
+  double* partials = nullptr;    // [kWindow][n_tiles][3], or [kWindow][n_tiles][units][3] (nodewise)
   double* chunk_sums = nullptr;  // [kWindow][n_chunks][3]
   unsigned* counters = nullptr;  // [kWindow]
   double* ring = nullptr;
@@ -227,6 +227,7 @@ struct vplbm_solver {
   int64_t me_read = 0;  // first step not yet returned by vplbm_momentum_exchange_forces
   int64_t me_stop = 0;  // step at which recording last stopped
 
+  bool nodewise = false;  // single steps run one node per thread
   int tiles_x = 0, tiles_y = 0, n_tiles = 0;
   StepParams base{};  // constants; src/dst/t/bodies filled per step
 
@@ -629,6 +630,13 @@ ReduceArgs reduce_args(const vplbm_solver* s, int64_t t0, int64_t steps) {
   a.steps = steps;
   a.ring_len = s->cfg.force_ring_len;
   a.reduce_mass = s->base.reduce_mass;
+  a.units = s->nodewise ? warps_per_block(s->cfg.storage) : 0;
+  a.f64 = s->cfg.storage == kF64;
+  a.nx = s->cfg.nx;
+  a.ny = s->cfg.ny;
+  a.tile_x = tile_x(s->cfg.storage);
+  a.tile_y = s->base.tile_y;
+  a.tiles_x = s->tiles_x;
   return a;
 }
 
@@ -638,6 +646,14 @@ cudaError_t launch_reduce(const ReduceArgs& a, cudaStream_t st) {
 
 cudaError_t launch_fused(const vplbm_solver* s, const StepParams& p) {
   const int coll = p.collision;
+  if (s->nodewise) {
+    switch (s->cfg.storage) {
+      case kF64: return launch_node_f64(coll, p, s->stream);
+      case kF32: return launch_node_f32(coll, p, s->stream);
+      case kF16: return launch_node_f16(coll, p, s->stream);
+      default: return launch_node_bf16(coll, p, s->stream);
+    }
+  }
   switch (s->cfg.storage) {
     case kF64: return launch_fused_f64(coll, p, s->stream);
     case kF32: return launch_fused_f32(coll, p, s->stream);
@@ -782,9 +798,22 @@ void tiles_of(const vplbm_config* c, int* tx, int* ty, int* nt) {
   *nt = *tx * *ty;
 }
 
-// Reduction scratch of a solver: a window of tile partials, their chunk sums
-// and the arrival counters.
-size_t partials_bytes(int nt) { return 3 * sizeof(double) * size_t(kWindow) * size_t(nt); }
+// Whether the solver's own steps run one node per thread (vplbm_node.cuh):
+// grids up to the size where the vector kernel catches up (measured there;
+// FP64 gains at every size, but a window of its record units takes 6 to 24
+// bytes a node, so larger grids keep a partial per tile).
+bool nodewise_rule(const vplbm_config* c) {
+  const int rows = tile_rows_of(c) / warps_per_block(c->storage);
+  if (tile_x(c->storage) * rows > kNodeThreads) return false;
+  const long long nodes = (long long)c->nx * c->ny;
+  return nodes <= (c->storage == kF64 ? 1ll << 23 : c->storage == kF32 ? 500000 : 420000);
+}
+
+// Reduction scratch of a solver: a window of partials per tile or record unit,
+// their chunk sums and the arrival counters.
+size_t partials_bytes(const vplbm_config* c, int nt) {
+  return 3 * sizeof(double) * size_t(kWindow) * size_t(nt) * (nodewise_rule(c) ? warps_per_block(c->storage) : 1);
+}
 size_t chunk_sums_bytes(int nt) { return 3 * sizeof(double) * size_t(kWindow) * size_t(reduce_chunks(nt)); }
 size_t counters_bytes() { return sizeof(unsigned) * size_t(kWindow); }
 
@@ -855,7 +884,7 @@ size_t vplbm_footprint_bytes(const vplbm_config* c) {
   size_t b = (aa ? 1 : 2) * 9 * plane * element_size(c->storage);  // A/B or in-place populations
   if (aa && c->bc_x != VPLBM_BC_PERIODIC) b += 9 * size_t(c->ny) * element_size(c->storage);
   b += plane;                                            // mask
-  b += partials_bytes(nt) + chunk_sums_bytes(nt) + counters_bytes();  // reduction scratch
+  b += partials_bytes(c, nt) + chunk_sums_bytes(nt) + counters_bytes();  // reduction scratch
   b += 3 * sizeof(double) * size_t(c->force_ring_len);
   b += sizeof(int) + sizeof(kEmptyBox);                  // error flag, static solid box
   if (c->bc_x == VPLBM_BC_INLET_CONVECTIVE) b += 2 * 3 * size_t(c->ny) * ghost_elem(c->storage);
@@ -905,10 +934,11 @@ vplbm_status vplbm_create(const vplbm_config* cfg, vplbm_solver** out) {
   cudaError_t e = cudaSuccess;
   cudaStream_t st0 = s->stream;
   s->aa = cfg->streaming == VPLBM_STREAM_AA;
+  s->nodewise = nodewise_rule(cfg);
   if ((st = mem_get(s, &s->f[0], pop)) != VPLBM_OK ||
       (!s->aa && (st = mem_get(s, &s->f[1], pop)) != VPLBM_OK) ||
       (st = mem_get(s, &s->mask, size_t(s->plane))) != VPLBM_OK ||
-      (st = mem_get(s, &s->partials, partials_bytes(s->n_tiles))) != VPLBM_OK ||
+      (st = mem_get(s, &s->partials, partials_bytes(cfg, s->n_tiles))) != VPLBM_OK ||
       (st = mem_get(s, &s->chunk_sums, chunk_sums_bytes(s->n_tiles))) != VPLBM_OK ||
       (st = mem_get(s, &s->counters, counters_bytes())) != VPLBM_OK ||
       (st = mem_get(s, &s->ring, 3 * sizeof(double) * cfg->force_ring_len)) != VPLBM_OK ||
@@ -1069,7 +1099,7 @@ vplbm_status vplbm_step(vplbm_solver* s, int64_t n) {
   for (int64_t k = 0; k < n; ++k) {
     if ((st = ensure_mask(s, s->t)) != VPLBM_OK) return st;
     StepParams p = step_params(s, s->t, 0);
-    p.partials += 3 * (long long)s->n_tiles * window;
+    p.partials += 3 * (long long)s->n_tiles * (s->nodewise ? warps_per_block(s->cfg.storage) : 1) * window;
     if (s->me_on) {
       VP_CUDA(s, launch_momentum_exchange(s, p, s->me_ring + 2 * (s->t % s->cfg.force_ring_len)));
       s->launches++;
@@ -1535,6 +1565,7 @@ vplbm_status vplbm_group_step(vplbm_solver* const* solvers, int32_t n, const int
         hp.push_back(step_params(s, s->t, 1));
         for (int tile = 0; tile < s->n_tiles; ++tile) ht.push_back(GroupTile{int(j), tile});
         hr.push_back(reduce_args(s, s->t, mem[j].steps));
+        hr.back().units = 0;  // the grouped kernel writes a partial per tile
         pl.max_chunks = std::max(pl.max_chunks, reduce_chunks(s->n_tiles));
         pl.prefix_steps.push_back(mem[j].steps);
         pl.prefix_tiles.push_back(int(ht.size()));

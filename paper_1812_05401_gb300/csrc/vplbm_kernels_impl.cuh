@@ -2,6 +2,7 @@
 // and defines its launchers.
 #include "vplbm_device.cuh"
 #include "vplbm_launch.h"
+#include "vplbm_node.cuh"
 
 #define VPLBM_CAT2(a, b) a##b
 #define VPLBM_CAT(a, b) VPLBM_CAT2(a, b)
@@ -25,6 +26,18 @@ static cudaError_t launch_fused_coll(const StepParams& p, cudaStream_t st) {
 
 cudaError_t VPLBM_FN(launch_fused_)(int coll, const StepParams& p, cudaStream_t st) {
   return coll == kTrt ? launch_fused_coll<kTrt>(p, st) : launch_fused_coll<kMrt>(p, st);
+}
+
+template <int COLL>
+static cudaError_t launch_node_coll(const StepParams& p, cudaStream_t st) {
+  const dim3 grid(p.n_tiles * warps_per_block(VPLBM_STORE)), blk(tile_x(VPLBM_STORE) * p.rows_per_warp);
+  if (p.mode == kModeAAPush) return launch_pdl(node_step_kernel<VPLBM_STORE, COLL, kModeAAPush>, grid, blk, st, p);
+  if (p.mode == kModeAALocal) return launch_pdl(node_step_kernel<VPLBM_STORE, COLL, kModeAALocal>, grid, blk, st, p);
+  return launch_pdl(node_step_kernel<VPLBM_STORE, COLL, kModeAB>, grid, blk, st, p);
+}
+
+cudaError_t VPLBM_FN(launch_node_)(int coll, const StepParams& p, cudaStream_t st) {
+  return coll == kTrt ? launch_node_coll<kTrt>(p, st) : launch_node_coll<kMrt>(p, st);
 }
 
 cudaError_t VPLBM_FN(launch_group_)(const StepParams* d_params, const GroupTile* d_table,

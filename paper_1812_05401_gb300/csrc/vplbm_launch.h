@@ -27,6 +27,7 @@ cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, cudaStr
 
 #define VPLBM_DECLARE_LAUNCHERS(SUFFIX)                                                         \
   cudaError_t launch_fused_##SUFFIX(int coll, const StepParams& p, cudaStream_t st);            \
+  cudaError_t launch_node_##SUFFIX(int coll, const StepParams& p, cudaStream_t st);             \
   cudaError_t launch_group_##SUFFIX(const StepParams* d_params,                                 \
                                     const GroupTile* d_table, int n_blocks, long long k,         \
                                     int mode, cudaStream_t st);                                 \

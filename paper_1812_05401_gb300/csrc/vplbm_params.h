@@ -57,6 +57,11 @@ __host__ __device__ constexpr int min_blocks_per_sm(int storage) {
 __host__ __device__ constexpr int npt(int storage) { return storage == kF64 ? 2 : 4; }
 __host__ __device__ constexpr int tile_x(int storage) { return kLanes * npt(storage); }
 
+// One-node-per-thread step (vplbm_node.cuh): threads of its largest block (a
+// record unit: tile_x x rows_per_warp nodes) and resident blocks.
+constexpr int kNodeThreads = 256;
+constexpr int kNodeBlocks = 4;
+
 // Block shape of the per-node kernels (initialisation, moments, import/export).
 constexpr int kBlockX = 64;
 constexpr int kBlockY = 4;
@@ -121,7 +126,9 @@ struct StepParams {
   long long plane;          // pitch * ny
   Consts<double> cd;        // constants for the FP64 kernels
   Consts<float> cf;         // the same, rounded, for the FP32 kernels
-  double* partials;         // [n_tiles][3] of this step (grouped: [kWindow][n_tiles][3])
+  // [n_tiles][3] of this step (grouped: [kWindow][n_tiles][3]; one node per
+  // thread: [n_tiles][warps_per_block][3], the tile's record units)
+  double* partials;
   int* flag;                // set to 1 on divergence
   long long t;              // index of this step
   int reduce_mass;
@@ -153,6 +160,11 @@ struct ReduceArgs {
   long long t0;            // step index of the window's first step
   long long steps;         // steps of the window (grouped: of the member's whole call)
   int n_tiles, ring_len, reduce_mass;
+  // 0: a partial per tile. Otherwise the partials are per record unit (this
+  // many a tile, rows of the tile by warp) and the tile's sum is formed here,
+  // as the vector kernel forms it: densities in FP32 or (f64) FP64
+  int units, f64;
+  int nx, ny, tile_x, tile_y, tiles_x;
 };
 
 // Arguments of the momentum-exchange reduction: a box of candidate solid

@@ -50,6 +50,30 @@ __device__ __forceinline__ void block_sum3(double v[3], double (*sm)[3]) {
   __syncthreads();
 }
 
+// Tile i's partial of a step.
+__device__ __forceinline__ void tile_partial(const ReduceArgs& a, const double* src, int i, double v[3]) {
+  if (!a.units) {
+    for (int k = 0; k < 3; ++k) v[k] = __ldcg(src + 3ll * i + k);
+    return;
+  }
+  const double* u = src + 3ll * i * a.units;
+  double m64 = 0.0;
+  float m32 = 0.f;
+  v[0] = v[1] = 0.0;
+  for (int w = 0; w < a.units; ++w) {
+    v[0] += __ldcg(u + 3 * w + 0);
+    v[1] += __ldcg(u + 3 * w + 1);
+    const double m = __ldcg(u + 3 * w + 2);
+    if (a.f64)
+      m64 += m;
+    else
+      m32 += float(m);
+  }
+  const int x0 = i % a.tiles_x * a.tile_x, y0 = i / a.tiles_x * a.tile_y;
+  // sum rho = active nodes + sum drho
+  v[2] = double(min(a.tile_x, a.nx - x0) * min(a.tile_y, a.ny - y0)) + (a.f64 ? m64 : double(m32));
+}
+
 // Records of the steps of one window: block (x, y) adds the partials of chunk
 // y of step x's tiles (each thread its strided share in increasing order,
 // then the block in a fixed order); with more than one chunk, the step's last
@@ -65,14 +89,16 @@ __device__ __forceinline__ void reduce_steps(const ReduceArgs& a, int step, int 
                                              int* s_last) {
   const int tid = threadIdx.x;
   const int n_chunks = reduce_chunks(a.n_tiles);
-  const double* src = a.partials + 3ll * a.n_tiles * step;
+  const double* src = a.partials + 3ll * a.n_tiles * (a.units ? a.units : 1) * step;
   const int end = min(a.n_tiles, (chunk + 1) * kChunkTiles);
   double v[3] = {0.0, 0.0, 0.0};
-#pragma unroll 4
+#pragma unroll 2
   for (int i = chunk * kChunkTiles + tid; i < end; i += kThreads) {
-    v[0] += __ldcg(src + 3ll * i + 0);
-    v[1] += __ldcg(src + 3ll * i + 1);
-    v[2] += __ldcg(src + 3ll * i + 2);
+    double t[3];
+    tile_partial(a, src, i, t);
+    v[0] += t[0];
+    v[1] += t[1];
+    v[2] += t[2];
   }
   block_sum3(v, sm);
   if (n_chunks > 1) {
