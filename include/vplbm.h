@@ -148,8 +148,8 @@ typedef struct {
    * stream). When set, every device buffer the solver owns comes from
    * dev_alloc(bytes, alloc_ctx) and goes back through dev_free(ptr,
    * alloc_ctx): the populations, mask, reduction scratch and rings at
-   * vplbm_create, the solid-velocity and momentum-exchange buffers when first
-   * needed, and the staging buffers of host transfers. dev_alloc returns
+   * vplbm_create, the solid-velocity, momentum-exchange and small grids'
+   * record buffers when first needed, and the staging buffers of host transfers. dev_alloc returns
    * memory on the current device, aligned to 256 bytes and ready for work
    * queued afterwards on the solver's stream (PyTorch's caching allocator on
    * that stream qualifies), or NULL when it has none: the call then fails
@@ -185,7 +185,9 @@ double vplbm_tau_from_reynolds(double u_ref, double l_ref, double re);
 /* Device bytes a solver with this configuration allocates at creation
  * (admission). Buffers taken later come on top when used: the static
  * solid-velocity field, the momentum-exchange records, the staging buffers
- * of host transfers. 0 for an invalid configuration. */
+ * of host transfers, and on small grids, with a call of many steps, the
+ * records of up to 64 of them (12 bytes a node for FP32). 0 for an invalid
+ * configuration. */
 size_t vplbm_footprint_bytes(const vplbm_config* cfg);
 
 /* Allocates the solver and sets the store to f*(0) = f_eq(rho0, u0) with an

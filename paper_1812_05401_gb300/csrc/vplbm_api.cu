@@ -206,7 +206,8 @@ struct vplbm_solver {
   int cur = 0;  // buffer holding f*(t)
   uint8_t* mask = nullptr;
   void* us = nullptr;
-  double* partials = nullptr;    // [kWindow][n_tiles][3], or [kWindow][n_tiles][units][3] (nodewise)
+  double* partials = nullptr;    // [kWindow][n_tiles][3], or as many steps of record units (nodewise)
+  double* unit_records = nullptr;  // nodewise, longer calls: [kWindow][n_tiles][units][3]
   double* chunk_sums = nullptr;  // [kWindow][n_chunks][3]
   unsigned* counters = nullptr;  // [kWindow]
   double* ring = nullptr;
@@ -228,6 +229,7 @@ struct vplbm_solver {
   int64_t me_stop = 0;  // step at which recording last stopped
 
   bool nodewise = false;  // single steps run one node per thread
+  bool units_refused = false;  // no memory for unit_records
   int tiles_x = 0, tiles_y = 0, n_tiles = 0;
   StepParams base{};  // constants; src/dst/t/bodies filled per step
 
@@ -621,7 +623,7 @@ StepParams step_params(const vplbm_solver* s, int64_t t, int parity) {
 
 ReduceArgs reduce_args(const vplbm_solver* s, int64_t t0, int64_t steps) {
   ReduceArgs a{};
-  a.partials = s->partials;
+  a.partials = s->unit_records ? s->unit_records : s->partials;
   a.chunk_sums = s->chunk_sums;
   a.counters = s->counters;
   a.ring = s->ring;
@@ -809,13 +811,30 @@ bool nodewise_rule(const vplbm_config* c) {
   return nodes <= (c->storage == kF64 ? 1ll << 23 : c->storage == kF32 ? 500000 : 420000);
 }
 
-// Reduction scratch of a solver: a window of partials per tile or record unit,
-// their chunk sums and the arrival counters.
-size_t partials_bytes(const vplbm_config* c, int nt) {
-  return 3 * sizeof(double) * size_t(kWindow) * size_t(nt) * (nodewise_rule(c) ? warps_per_block(c->storage) : 1);
-}
+// Reduction scratch of a solver: a window of tile partials, their chunk sums
+// and the arrival counters.
+size_t partials_bytes(int nt) { return 3 * sizeof(double) * size_t(kWindow) * size_t(nt); }
 size_t chunk_sums_bytes(int nt) { return 3 * sizeof(double) * size_t(kWindow) * size_t(reduce_chunks(nt)); }
 size_t counters_bytes() { return sizeof(unsigned) * size_t(kWindow); }
+
+// Steps whose records the scratch holds. One node per thread writes several
+// record units a tile: the tiles' scratch then holds a few steps, and calls of
+// more steps take a window of units (12 bytes a node for FP32) when first made,
+// so that the sums' launch (about 2 us) stays a small part of their steps
+// (1024 x 256 FP32 6.0 -> 5.2 us per step). Not while the stream captures a
+// graph, where an allocation would belong to the graph; without the memory the
+// window stays short.
+int step_window(vplbm_solver* s, int64_t n) {
+  if (!s->nodewise) return kWindow;
+  const int units = warps_per_block(s->cfg.storage);
+  const int few = kWindow / units;
+  if (n > few && !s->unit_records && !s->units_refused) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s->stream, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone)
+      s->units_refused = mem_get(s, &s->unit_records, partials_bytes(s->n_tiles) * units) != VPLBM_OK;
+  }
+  return s->unit_records ? kWindow : few;
+}
 
 vplbm_status check_usable(vplbm_solver* s) {
   if (!s) return VPLBM_ERR_INVALID;
@@ -884,7 +903,7 @@ size_t vplbm_footprint_bytes(const vplbm_config* c) {
   size_t b = (aa ? 1 : 2) * 9 * plane * element_size(c->storage);  // A/B or in-place populations
   if (aa && c->bc_x != VPLBM_BC_PERIODIC) b += 9 * size_t(c->ny) * element_size(c->storage);
   b += plane;                                            // mask
-  b += partials_bytes(c, nt) + chunk_sums_bytes(nt) + counters_bytes();  // reduction scratch
+  b += partials_bytes(nt) + chunk_sums_bytes(nt) + counters_bytes();  // reduction scratch
   b += 3 * sizeof(double) * size_t(c->force_ring_len);
   b += sizeof(int) + sizeof(kEmptyBox);                  // error flag, static solid box
   if (c->bc_x == VPLBM_BC_INLET_CONVECTIVE) b += 2 * 3 * size_t(c->ny) * ghost_elem(c->storage);
@@ -938,7 +957,7 @@ vplbm_status vplbm_create(const vplbm_config* cfg, vplbm_solver** out) {
   if ((st = mem_get(s, &s->f[0], pop)) != VPLBM_OK ||
       (!s->aa && (st = mem_get(s, &s->f[1], pop)) != VPLBM_OK) ||
       (st = mem_get(s, &s->mask, size_t(s->plane))) != VPLBM_OK ||
-      (st = mem_get(s, &s->partials, partials_bytes(cfg, s->n_tiles))) != VPLBM_OK ||
+      (st = mem_get(s, &s->partials, partials_bytes(s->n_tiles))) != VPLBM_OK ||
       (st = mem_get(s, &s->chunk_sums, chunk_sums_bytes(s->n_tiles))) != VPLBM_OK ||
       (st = mem_get(s, &s->counters, counters_bytes())) != VPLBM_OK ||
       (st = mem_get(s, &s->ring, 3 * sizeof(double) * cfg->force_ring_len)) != VPLBM_OK ||
@@ -1095,10 +1114,13 @@ vplbm_status vplbm_step(vplbm_solver* s, int64_t n) {
   if (st != VPLBM_OK) return st;
   if (n < 0) return fail(s, VPLBM_ERR_INVALID, "n must be >= 0");
   TraceRange trace("vplbm_step");
-  int64_t window = 0;  // steps whose tile partials await their sum
+  const int most = step_window(s, n);
+  if (s->sticky) return VPLBM_ERR_CUDA;
+  int64_t window = 0;  // steps whose partials await their sum
   for (int64_t k = 0; k < n; ++k) {
     if ((st = ensure_mask(s, s->t)) != VPLBM_OK) return st;
     StepParams p = step_params(s, s->t, 0);
+    if (s->unit_records) p.partials = s->unit_records;
     p.partials += 3 * (long long)s->n_tiles * (s->nodewise ? warps_per_block(s->cfg.storage) : 1) * window;
     if (s->me_on) {
       VP_CUDA(s, launch_momentum_exchange(s, p, s->me_ring + 2 * (s->t % s->cfg.force_ring_len)));
@@ -1118,7 +1140,7 @@ vplbm_status vplbm_step(vplbm_solver* s, int64_t n) {
     s->launches++;
     s->cur ^= 1;
     s->t++;
-    if (++window == kWindow || k == n - 1) {
+    if (++window == most || k == n - 1) {
       VP_CUDA(s, launch_reduce(reduce_args(s, s->t - window, window), s->stream));
       window = 0;
     }
@@ -1566,6 +1588,7 @@ vplbm_status vplbm_group_step(vplbm_solver* const* solvers, int32_t n, const int
         for (int tile = 0; tile < s->n_tiles; ++tile) ht.push_back(GroupTile{int(j), tile});
         hr.push_back(reduce_args(s, s->t, mem[j].steps));
         hr.back().units = 0;  // the grouped kernel writes a partial per tile
+        hr.back().partials = s->partials;
         pl.max_chunks = std::max(pl.max_chunks, reduce_chunks(s->n_tiles));
         pl.prefix_steps.push_back(mem[j].steps);
         pl.prefix_tiles.push_back(int(ht.size()));
@@ -1669,7 +1692,8 @@ void vplbm_destroy(vplbm_solver* s) {
   if (s->stream) {
     void* bufs[] = {s->f[0], s->aa ? nullptr : s->f[1], s->mask, s->us, s->partials, s->chunk_sums,
                     s->counters, s->ring, s->flag, s->static_box, s->me_ring,
-                    s->me_scratch, s->me_counter, s->ghost[0], s->ghost[1], s->z, s->lost};
+                    s->me_scratch, s->me_counter, s->ghost[0], s->ghost[1], s->z, s->lost,
+                    s->unit_records};
     if (s->cfg.dev_free) cudaStreamSynchronize(s->stream);  // once, for all of them
     for (void* b : bufs) {
       if (!b) continue;
