@@ -185,8 +185,9 @@ double vplbm_tau_from_reynolds(double u_ref, double l_ref, double re);
 /* Device bytes a solver with this configuration allocates at creation
  * (admission). Buffers taken later come on top when used: the static
  * solid-velocity field, the momentum-exchange records, the staging buffers
- * of host transfers, and on small grids, with a call of many steps, the
- * records of up to 64 of them (12 bytes a node for FP32). 0 for an invalid
+ * of host transfers, on small grids, with a call of many steps, the
+ * records of up to 64 of them (12 bytes a node for FP32), and, where steps run
+ * in pairs, a second mask for moving bodies (1 byte a node). 0 for an invalid
  * configuration. */
 size_t vplbm_footprint_bytes(const vplbm_config* cfg);
 
@@ -223,7 +224,9 @@ vplbm_status vplbm_set_mask_and_solid_velocity(vplbm_solver* s, const uint8_t* c
 vplbm_status vplbm_set_bodies(vplbm_solver* s, const vplbm_body* bodies, int32_t n);
 
 /* Advances n >= 0 time steps (asynchronous). Step t maps f*(t) to f*(t+1)
- * with the mask and solid velocity of time t. */
+ * with the mask and solid velocity of time t. On FP32 A/B grids of more than
+ * 4,000,000 nodes (SRT or two-rate MRT, no momentum exchange) consecutive
+ * steps of a call run two a launch, with the results of single steps. */
 vplbm_status vplbm_step(vplbm_solver* s, int64_t n);
 
 /* Waits for the solver's stream and reports VPLBM_ERR_DIVERGED if any step
@@ -314,15 +317,15 @@ vplbm_status vplbm_momentum_exchange_forces(vplbm_solver* s, double* fx, double*
 vplbm_status vplbm_group_step(vplbm_solver* const* solvers, int32_t n,
                               const int64_t* steps);
 
-/* Kernel launches this solver issued on its hot path (fused steps and mask
- * updates; the sums of step records, one per up to 64 steps of a call, are not
+/* Kernel launches this solver issued on its hot path (fused steps, one launch
+ * for two where they run in pairs, and mask updates; the sums of step records, one per up to 64 steps of a call, are not
  * counted) since creation. */
 int64_t vplbm_launch_count(const vplbm_solver* s);
 
 /* Timing of the fused step kernel: enable = 1 brackets each fused launch with
  * CUDA events on the solver's stream. vplbm_fused_timing synchronizes and
- * returns the summed device time (ms) and the number of timed launches since
- * the last read. */
+ * returns the summed device time (ms) and the number of steps the timed
+ * launches made since the last read. */
 vplbm_status vplbm_enable_timing(vplbm_solver* s, int32_t enable);
 vplbm_status vplbm_fused_timing(vplbm_solver* s, double* total_ms, int64_t* launches);
 

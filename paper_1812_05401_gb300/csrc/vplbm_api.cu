@@ -194,6 +194,12 @@ int row_pitch(int nx, int storage) {
 
 }  // namespace
 
+// A timed launch of the fused step and the steps it made.
+struct TimedLaunch {
+  cudaEvent_t first, second;
+  int steps;
+};
+
 struct vplbm_solver {
   vplbm_config cfg{};
   int pitch = 0;
@@ -237,12 +243,15 @@ struct vplbm_solver {
   int64_t ring_read = 0;  // first step not yet returned by vplbm_forces
   std::vector<vplbm_body> bodies;
   bool moving = false;
+  bool pair = false;             // consecutive steps run two a launch (vplbm_pair.cuh)
+  uint8_t* mask_next = nullptr;  // pair, moving bodies: the mask of a pair's second step
+  int64_t mask_next_t = -1;      // time it reflects (-1: not a copy of the mask's static layer)
   int64_t mask_t = -1;  // time the moving bodies' mask reflects (-1: none)
 
   int64_t launches = 0;
   bool timing = false;
   std::vector<cudaEvent_t> ev_pool;
-  std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev_pending;
+  std::vector<TimedLaunch> ev_pending;
   double timed_ms = 0.0;
   int64_t timed_count = 0;
 
@@ -392,7 +401,7 @@ Box unite(Box a, Box b) {
   return Box{std::min(a.x0, b.x0), std::min(a.y0, b.y0), std::max(a.x1, b.x1), std::max(a.y1, b.y1)};
 }
 
-vplbm_status launch_mask_update(vplbm_solver* s, Box box, int64_t t) {
+vplbm_status launch_mask_update(vplbm_solver* s, uint8_t* mask, Box box, int64_t t) {
   if (box.empty()) return VPLBM_OK;
   BodyGeomSet g{};
   g.n = int(s->bodies.size());
@@ -406,26 +415,39 @@ vplbm_status launch_mask_update(vplbm_solver* s, Box box, int64_t t) {
   }
   const dim3 blk(64, 4);
   const int w = box.x1 - box.x0 + 1, h = box.y1 - box.y0 + 1;
-  VP_CUDA(s, launch_pdl(mask_update_kernel, grid2d(w, h, blk), blk, s->stream, s->mask, s->pitch, box.x0,
+  VP_CUDA(s, launch_pdl(mask_update_kernel, grid2d(w, h, blk), blk, s->stream, mask, s->pitch, box.x0,
                         box.y0, w, h, g));
   s->launches++;
   return VPLBM_OK;
 }
 
-// Brings the mask of the moving bodies to time t (only the swept region).
-vplbm_status ensure_mask(vplbm_solver* s, int64_t t) {
-  if (!s->moving || s->mask_t == t) return VPLBM_OK;
+// Brings a mask of the moving bodies from time *mask_t (-1: unknown) to time t
+// (only the swept region).
+vplbm_status ensure_mask(vplbm_solver* s, uint8_t* mask, int64_t* mask_t, int64_t t) {
+  if (!s->moving || *mask_t == t) return VPLBM_OK;
   Box box{0, 0, -1, -1};
   for (const auto& b : s->bodies) {
     if (b.period <= 0.0) continue;
     box = unite(box, body_box(s, b, t));
-    if (s->mask_t >= 0) box = unite(box, body_box(s, b, s->mask_t));
+    if (*mask_t >= 0) box = unite(box, body_box(s, b, *mask_t));
   }
-  if (s->mask_t < 0) box = Box{0, 0, s->cfg.nx - 1, s->cfg.ny - 1};
-  vplbm_status st = launch_mask_update(s, box, t);
+  if (*mask_t < 0) box = Box{0, 0, s->cfg.nx - 1, s->cfg.ny - 1};
+  vplbm_status st = launch_mask_update(s, mask, box, t);
   if (st != VPLBM_OK) return st;
-  s->mask_t = t;
+  *mask_t = t;
   return VPLBM_OK;
+}
+vplbm_status ensure_mask(vplbm_solver* s, int64_t t) { return ensure_mask(s, s->mask, &s->mask_t, t); }
+
+// The second step's mask of a pair of steps t, t + 1 whose bodies move (the
+// first step's is at t): taken over from the first's where that was rewritten
+// since, then moved on like it.
+vplbm_status ensure_next_mask(vplbm_solver* s, int64_t t) {
+  if (s->mask_next_t < 0) {
+    VP_CUDA(s, cudaMemcpyAsync(s->mask_next, s->mask, size_t(s->plane), cudaMemcpyDeviceToDevice, s->stream));
+    s->mask_next_t = t;
+  }
+  return ensure_mask(s, s->mask_next, &s->mask_next_t, t + 1);
 }
 
 // Resets the static solid layer's box to empty and recomputes it from the
@@ -792,6 +814,19 @@ int tile_rows_of(const vplbm_config* c) {
   return rows;
 }
 
+// Whether a solver's consecutive steps run two a launch (vplbm_pair.cuh): FP32
+// grids whose populations exceed L2 (2 x 144 MB at the line). Per step, single
+// against paired: 2896 x 1448 49.6 / 45.8 us, 4096 x 1024 51.7 / 45.2, 6048 x
+// 2016 150 / 133, 16384 x 4096 773 / 625; below, L2 holds much of what a pair
+// saves: 2048 x 1024 25.8 / 26.3, 1001 x 1401 18.6 / 22.0.
+constexpr long long kPairNodes = 4000000;
+bool pair_rule(const vplbm_config* c) {
+  StepParams consts{};
+  physics_consts(c, &consts);
+  return c->storage == VPLBM_F32 && c->streaming == VPLBM_STREAM_AB && tile_rows_of(c) % kPairRows == 0 &&
+         (long long)c->nx * c->ny > kPairNodes && consts.collision == kTrt;
+}
+
 void tiles_of(const vplbm_config* c, int* tx, int* ty, int* nt) {
   const int tw = tile_x(c->storage);
   const int rows = tile_rows_of(c);
@@ -848,7 +883,7 @@ vplbm_status drain_timing(vplbm_solver* s) {
     VP_CUDA(s, cudaEventSynchronize(pr.second));
     VP_CUDA(s, cudaEventElapsedTime(&ms, pr.first, pr.second));
     s->timed_ms += ms;
-    s->timed_count++;
+    s->timed_count += pr.steps;
     s->ev_pool.push_back(pr.first);
     s->ev_pool.push_back(pr.second);
   }
@@ -954,6 +989,8 @@ vplbm_status vplbm_create(const vplbm_config* cfg, vplbm_solver** out) {
   cudaStream_t st0 = s->stream;
   s->aa = cfg->streaming == VPLBM_STREAM_AA;
   s->nodewise = nodewise_rule(cfg);
+  s->pair = pair_rule(cfg);
+  if (s->pair && (e = prepare_pair_f32()) != cudaSuccess) return bail(cuda_fail(s, e, "prepare_pair"));
   if ((st = mem_get(s, &s->f[0], pop)) != VPLBM_OK ||
       (!s->aa && (st = mem_get(s, &s->f[1], pop)) != VPLBM_OK) ||
       (st = mem_get(s, &s->mask, size_t(s->plane))) != VPLBM_OK ||
@@ -1064,6 +1101,7 @@ vplbm_status vplbm_set_mask_and_solid_velocity(vplbm_solver* s, const uint8_t* c
     }
   }
   const dim3 blk(64, 4);
+  s->mask_next_t = -1;
   mask_import_kernel<<<grid2d(nx, ny, blk), blk, 0, s->stream>>>(s->mask, s->pitch, nx, ny, dchi);
   VP_CUDA(s, cudaGetLastError());
   if ((st = update_static_box(s)) != VPLBM_OK) return st;
@@ -1083,7 +1121,7 @@ vplbm_status vplbm_set_mask_and_solid_velocity(vplbm_solver* s, const uint8_t* c
   }
   // Rebuild the bodies where the static layer changed.
   if (!s->bodies.empty()) {
-    st = launch_mask_update(s, Box{0, 0, nx - 1, ny - 1}, s->t);
+    st = launch_mask_update(s, s->mask, Box{0, 0, nx - 1, ny - 1}, s->t);
     if (st != VPLBM_OK) return st;
     s->mask_t = s->moving ? s->t : -1;
   }
@@ -1099,13 +1137,17 @@ vplbm_status vplbm_set_bodies(vplbm_solver* s, const vplbm_body* bodies, int32_t
     if (!(bodies[i].radius >= 0.0) || !std::isfinite(bodies[i].cx) || !std::isfinite(bodies[i].cy))
       return fail(s, VPLBM_ERR_INVALID, "body radius must be >= 0 and centre finite");
   s->bodies.assign(bodies, bodies + n);
+  s->mask_next_t = -1;
   s->moving = false;
   for (const auto& b : s->bodies)
     if (b.period > 0.0 && (b.amp_x != 0.0 || b.amp_y != 0.0)) s->moving = true;
   // Full rebuild at the current time (also clears removed bodies).
-  st = launch_mask_update(s, Box{0, 0, s->cfg.nx - 1, s->cfg.ny - 1}, s->t);
+  st = launch_mask_update(s, s->mask, Box{0, 0, s->cfg.nx - 1, s->cfg.ny - 1}, s->t);
   if (st != VPLBM_OK) return st;
   s->mask_t = s->moving ? s->t : -1;
+  // without memory for the second mask the steps run one a launch
+  if (s->pair && s->moving && !s->mask_next && mem_get(s, &s->mask_next, size_t(s->plane)) != VPLBM_OK && s->sticky)
+    return VPLBM_ERR_CUDA;
   return VPLBM_OK;
 }
 
@@ -1116,12 +1158,26 @@ vplbm_status vplbm_step(vplbm_solver* s, int64_t n) {
   TraceRange trace("vplbm_step");
   const int most = step_window(s, n);
   if (s->sticky) return VPLBM_ERR_CUDA;
+  const long long records = 3ll * s->n_tiles * (s->nodewise ? warps_per_block(s->cfg.storage) : 1);  // of a step
+  // momentum exchange reads the populations of every step
+  const bool pairs = s->pair && !s->me_on && (!s->moving || s->mask_next);
   int64_t window = 0;  // steps whose partials await their sum
-  for (int64_t k = 0; k < n; ++k) {
+  for (int64_t k = 0; k < n;) {
     if ((st = ensure_mask(s, s->t)) != VPLBM_OK) return st;
     StepParams p = step_params(s, s->t, 0);
     if (s->unit_records) p.partials = s->unit_records;
-    p.partials += 3 * (long long)s->n_tiles * (s->nodewise ? warps_per_block(s->cfg.storage) : 1) * window;
+    p.partials += records * window;
+    const int count = pairs && n - k >= 2 && window + 2 <= most ? 2 : 1;
+    PairParams pp;
+    if (count == 2) {
+      if (s->moving && (st = ensure_next_mask(s, s->t)) != VPLBM_OK) return st;
+      pp.a = pp.b = p;
+      pp.a.ghost_dst = nullptr;  // advanced once, by the second step
+      pp.b.t = s->t + 1;
+      pp.b.partials += records;
+      if (s->moving) pp.b.mask = s->mask_next;
+      fill_bodies(s, s->t + 1, &pp.b);
+    }
     if (s->me_on) {
       VP_CUDA(s, launch_momentum_exchange(s, p, s->me_ring + 2 * (s->t % s->cfg.force_ring_len)));
       s->launches++;
@@ -1132,15 +1188,17 @@ vplbm_status vplbm_step(vplbm_solver* s, int64_t n) {
       if ((st = get_event(s, &e1)) != VPLBM_OK) return st;
       VP_CUDA(s, cudaEventRecord(e0, s->stream));
     }
-    VP_CUDA(s, launch_fused(s, p));
+    VP_CUDA(s, count == 2 ? launch_pair_f32(pp, s->stream) : launch_fused(s, p));
     if (s->timing) {
       VP_CUDA(s, cudaEventRecord(e1, s->stream));
-      s->ev_pending.emplace_back(e0, e1);
+      s->ev_pending.push_back(TimedLaunch{e0, e1, count});
     }
     s->launches++;
     s->cur ^= 1;
-    s->t++;
-    if (++window == most || k == n - 1) {
+    s->t += count;
+    k += count;
+    window += count;
+    if (window == most || k == n) {
       VP_CUDA(s, launch_reduce(reduce_args(s, s->t - window, window), s->stream));
       window = 0;
     }
@@ -1371,6 +1429,7 @@ vplbm_status vplbm_load_state(vplbm_solver* s, const void* buf, size_t bytes) {
   const char* in = static_cast<const char*>(buf) + sizeof(h);
   VP_CUDA(s, cudaMemcpyAsync(s->f[s->cur], in, h.pop_bytes, cudaMemcpyHostToDevice, s->stream));
   in += h.pop_bytes;
+  s->mask_next_t = -1;
   VP_CUDA(s, cudaMemcpyAsync(s->mask, in, h.mask_bytes, cudaMemcpyHostToDevice, s->stream));
   in += h.mask_bytes;
   if (h.has_us) {
@@ -1693,7 +1752,7 @@ void vplbm_destroy(vplbm_solver* s) {
     void* bufs[] = {s->f[0], s->aa ? nullptr : s->f[1], s->mask, s->us, s->partials, s->chunk_sums,
                     s->counters, s->ring, s->flag, s->static_box, s->me_ring,
                     s->me_scratch, s->me_counter, s->ghost[0], s->ghost[1], s->z, s->lost,
-                    s->unit_records};
+                    s->unit_records, s->mask_next};
     if (s->cfg.dev_free) cudaStreamSynchronize(s->stream);  // once, for all of them
     for (void* b : bufs) {
       if (!b) continue;

@@ -301,7 +301,7 @@ __device__ __forceinline__ typename S::T outlet_ghost(const StepParams& p,
   const long long gi = (long long)(as == 3 ? 0 : (as == 6 ? 1 : 2)) * p.ny + ys;
   const T f_last = load_h<S>(p, src + (long long)as * p.plane + (long long)ys * p.pitch + (p.nx - 1), as);
   const T g = mul(mad(c.u_conv, f_last, static_cast<const T*>(p.ghost_src)[gi]), c.conv_inv);
-  if (write) static_cast<T*>(p.ghost_dst)[gi] = g;
+  if (write && p.ghost_dst) static_cast<T*>(p.ghost_dst)[gi] = g;
   return g;
 }
 
@@ -753,35 +753,48 @@ __device__ __forceinline__ void shift_row(int nx, int x0, int lane, const typena
   }
 }
 
+// The source row of direction a's population for row y of nodes.
+template <class S, bool GEN, bool AA = false>
+__device__ __forceinline__ const typename S::E* source_row(const StepParams& p, const typename S::E* src, int a,
+                                                           int y) {
+  int as = a, ys = y - cy(a);
+  if (GEN && (ys < 0 || ys >= p.ny)) {
+    if (p.bc_y == kBcPeriodic) {
+      ys = ys < 0 ? ys + p.ny : ys - p.ny;
+    } else {  // free slip: the mirror of the population that left this row
+      as = mirror_y(a);
+      ys = y;
+    }
+  }
+  return src + (long long)(AA ? opposite(as) : as) * p.plane + (long long)ys * p.pitch;
+}
+
+// The values a lane's N nodes xb .. xb + N - 1 of row y pull, by the column
+// they come from.
+template <class S, int N, bool GEN, bool AA = false>
+__device__ __forceinline__ void load_row(const StepParams& p, const typename S::E* src, int xb, int y,
+                                         bool lane_active, typename S::T (&v)[9][N]) {
+#pragma unroll
+  for (int a = 0; a < 9; ++a) {
+    const typename S::E* row = source_row<S, GEN, AA>(p, src, a, y);
+    if (!GEN || lane_active) {
+      S::load_h(row + xb, v[a], a);
+    } else {
+#pragma unroll
+      for (int k = 0; k < N; ++k) v[a][k] = typename S::T(0);
+    }
+  }
+}
+
 // The pulled populations of a lane's N nodes xb .. xb + N - 1 of row y.
 template <class S, int N, bool GEN, bool AA = false>
 __device__ __forceinline__ void pull_row(const StepParams& p, const typename S::E* src,
                                          const EdgeLane<S, kLanes * N, GEN, AA>& el, int x0, int y, int lane,
                                          bool lane_active, typename S::T (&h)[N][9]) {
   using T = typename S::T;
-  using E = typename S::E;
   const T edge = el.value(p, src, x0, y, lane);
-  const int xb = x0 + lane * N;
   T v[9][N];
-#pragma unroll
-  for (int a = 0; a < 9; ++a) {
-    int as = a, ys = y - cy(a);
-    if (GEN && (ys < 0 || ys >= p.ny)) {
-      if (p.bc_y == kBcPeriodic) {
-        ys = ys < 0 ? ys + p.ny : ys - p.ny;
-      } else {  // free slip: the mirror of the population that left this row
-        as = mirror_y(a);
-        ys = y;
-      }
-    }
-    const E* row = src + (long long)(AA ? opposite(as) : as) * p.plane + (long long)ys * p.pitch;
-    if (!GEN || lane_active) {
-      S::load_h(row + xb, v[a], a);
-    } else {
-#pragma unroll
-      for (int k = 0; k < N; ++k) v[a][k] = T(0);
-    }
-  }
+  load_row<S, N, GEN, AA>(p, src, x0 + lane * N, y, lane_active, v);
   shift_row<S, N, GEN>(p.nx, x0, lane, v, edge, h);
 }
 
@@ -999,10 +1012,11 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, int tx, int t
   return x0 >= 1 && x0 + tile_x(STORE) <= p.nx - 1 && y0 >= 1 && y0 + p.tile_y <= p.ny - 1;
 }
 
-// Whether fluid nodes of a tile take the force-free form of the step.
+// Whether fluid node (x, y) takes the force-free form of the step: those of
+// tiles that touch no boundary do.
 template <int STORE>
-__device__ __forceinline__ bool free_form(const StepParams& p, int tx, int ty) {
-  return p.force_free && interior_tile<STORE>(p, tx, ty);
+__device__ __forceinline__ bool free_form(const StepParams& p, int x, int y) {
+  return p.force_free && interior_tile<STORE>(p, x / tile_x(STORE), y / p.tile_y);
 }
 
 // Storages whose rows of fluid nodes are collided without branches: FP32, and
@@ -1012,7 +1026,9 @@ __host__ __device__ constexpr bool straight_rows(int storage) { return storage =
 
 // Collide one row's N pulled nodes of a lane whose first node lies in the
 // domain. free: fluid nodes take the force-free form (free_form of their tile).
-template <int STORE, int COLL, bool GEN, int N>
+// ONE: a lane's nodes one after the other, for kernels short of registers (the
+// paired step at 80 registers spills 216 bytes otherwise).
+template <int STORE, int COLL, bool GEN, int N, bool ONE = false>
 __device__ __forceinline__ void collide_row(const StepParams& p, typename Store<STORE>::T (&h)[N][9],
                                             unsigned mw, int xb, int y, bool free,
                                             RowSums<typename Store<STORE>::T>& acc) {
@@ -1039,6 +1055,7 @@ __device__ __forceinline__ void collide_row(const StepParams& p, typename Store<
     bool sound = true;
 #pragma unroll
     for (int k = 0; k < N; ++k) {
+      if (ONE && k > 0 && mw != 0) break;  // never: keeps the nodes' instructions apart
       const Macro<T> q = macros<T, FORM, REF>(p, h[k], 0, xb + k, y);
       collide_trt<T, FORM, REF>(p, h[k], q);
       sound = sound && q.rho > T(0) && q.rho < T(1e30);
@@ -1087,70 +1104,61 @@ __device__ __forceinline__ void round_words(const StepParams& p, int xb, int y, 
     nb[j] = sr ? round_bits(unsigned((long long)y * ((p.nx + 1) >> 1) + (xb >> 1) + j), key) : 0u;
 }
 
-// The tile's share of the records of K steps (reduce_kernel adds the tiles):
-// the force on the solid nodes, summed per thread in the arithmetic type (each
-// thread holds at most 16 nodes) and in FP64 from the thread up; the total
-// density, in the arithmetic type within the block and FP64 from the tile up.
-// Warps and blocks without solid nodes skip the FP64 work (on GB300 FP64 runs
-// at a small fraction of the FP32 rate).
-template <int STORE, int K>
-__device__ __forceinline__ void tile_records(const StepParams& p, int tile, int x0, int y0,
-                                             const RowSums<typename Store<STORE>::T> (&acc)[K],
-                                             double* const (&partials)[K]) {
+// A tile's share of a step's records (reduce_kernel adds the tiles): the force
+// on the solid nodes, summed per thread in the arithmetic type (each thread
+// holds at most 16 nodes) and in FP64 from the thread up; the total density, in
+// the arithmetic type within the block and FP64 from the tile up. Warps and
+// blocks without solid nodes skip the FP64 work (on GB300 FP64 runs at a small
+// fraction of the FP32 rate).
+template <int STORE>
+struct TileSums {  // in shared memory, by warp
+  double f[warps_per_block(STORE)][2];
+  typename Store<STORE>::T dm[warps_per_block(STORE)];
+};
+template <int STORE>
+__device__ __forceinline__ void warp_records(const StepParams& p, const RowSums<typename Store<STORE>::T>& acc,
+                                             TileSums<STORE>& sums) {
+  const bool warp_solid = __any_sync(0xffffffffu, acc.solid);
+  typename Store<STORE>::T dm = acc.dm;
+  double bfx = 0.0, bfy = 0.0;
+  if (p.reduce_mass) dm = warp_sum(dm);
+  if (warp_solid) {
+    bfx = warp_sum(double(acc.fx));
+    bfy = warp_sum(double(acc.fy));
+  }
+  if (threadIdx.x == 0) {
+    sums.dm[threadIdx.y] = dm;
+    sums.f[threadIdx.y][0] = bfx;
+    sums.f[threadIdx.y][1] = bfy;
+  }
+}
+// One thread, once every warp's sums stand (solid: whether any warp has solid nodes).
+template <int STORE>
+__device__ __forceinline__ void tile_record(const StepParams& p, int tile, int x0, int y0, bool solid,
+                                            const TileSums<STORE>& sums, double* partials) {
   using T = typename Store<STORE>::T;
   constexpr int W = warps_per_block(STORE);
   constexpr int TX = tile_x(STORE);
-  __shared__ double sm[K][W][2];
-  __shared__ T smass[K][W];
-  const int lane = threadIdx.x, warp = threadIdx.y;
-  const int tid = lane + warp * kLanes;
-  bool block_solid[K];
+  double ts[3] = {0.0, 0.0, 0.0};
+  T msum = T(0);
 #pragma unroll
-  for (int i = 0; i < K; ++i) {
-    const bool warp_solid = __any_sync(0xffffffffu, acc[i].solid);
-    T dm = acc[i].dm;
-    double bfx = 0.0, bfy = 0.0;
-    if (warp_solid) {
-      bfx = double(acc[i].fx);
-      bfy = double(acc[i].fy);
-    }
-    if (p.reduce_mass) dm = warp_sum(dm);
-    if (warp_solid) {
-      bfx = warp_sum(bfx);
-      bfy = warp_sum(bfy);
-    }
-    if (lane == 0) {
-      smass[i][warp] = dm;
-      sm[i][warp][0] = bfx;
-      sm[i][warp][1] = bfy;
-    }
-    block_solid[i] = __syncthreads_or(acc[i].solid);
-  }
-  if (tid == 0) {
+  for (int w = 0; w < W; ++w) msum += sums.dm[w];
+  if (solid) {
 #pragma unroll
-    for (int i = 0; i < K; ++i) {
-      double ts[3] = {0.0, 0.0, 0.0};
-      T msum = T(0);
-#pragma unroll
-      for (int w = 0; w < W; ++w) msum += smass[i][w];
-      if (block_solid[i]) {
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-          ts[0] += sm[i][w][0];
-          ts[1] += sm[i][w][1];
-        }
-      }
-      if (p.reduce_mass) {
-        // sum rho = active nodes + sum drho
-        const int nact = min(TX, p.nx - x0) * min(p.tile_y, p.ny - y0);
-        ts[2] = double(nact) + double(msum);
-      }
-      double* out = partials[i] + 3ll * tile;
-      out[0] = ts[0];
-      out[1] = ts[1];
-      out[2] = ts[2];
+    for (int w = 0; w < W; ++w) {
+      ts[0] += sums.f[w][0];
+      ts[1] += sums.f[w][1];
     }
   }
+  if (p.reduce_mass) {
+    // sum rho = active nodes + sum drho
+    const int nact = min(TX, p.nx - x0) * min(p.tile_y, p.ny - y0);
+    ts[2] = double(nact) + double(msum);
+  }
+  double* out = partials + 3ll * tile;
+  out[0] = ts[0];
+  out[1] = ts[1];
+  out[2] = ts[2];
 }
 
 // MODE: kModeAB (pull from p.src, store to p.dst), or one of the two in-place
@@ -1178,7 +1186,7 @@ __device__ __forceinline__ void step_tile(const StepParams& p, int tile, long lo
   E* dst = static_cast<E*>(p.dst);
   E* buf = static_cast<E*>(p.dst);  // the in-place modes' one buffer
 
-  RowSums<T> acc[1];
+  RowSums<T> acc;
   const unsigned key = round_bits(unsigned(t), p.round_key);
 
   // Collide and store one row of pulled populations (lane_active: the lane's
@@ -1188,7 +1196,7 @@ __device__ __forceinline__ void step_tile(const StepParams& p, int tile, long lo
     const long long i = (long long)y * p.pitch + xb;
     const unsigned mw = mask_word<N>(p.mask + i);
     const bool sr = S::kSixteen && p.stochastic;
-    collide_row<STORE, COLL, GEN>(p, h, mw, xb, y, !GEN && p.force_free, acc[0]);
+    collide_row<STORE, COLL, GEN>(p, h, mw, xb, y, !GEN && p.force_free, acc);
     unsigned nb[(N + 1) / 2];
     round_words(p, xb, y, key, sr, nb);
     if constexpr (MODE == kModeAB) {
@@ -1291,8 +1299,10 @@ __device__ __forceinline__ void step_tile(const StepParams& p, int tile, long lo
   }
 
   pdl_trigger();
-  double* const parts[1] = {partials};
-  tile_records<STORE>(p, tile, x0, y0, acc, parts);
+  __shared__ TileSums<STORE> sums;
+  warp_records<STORE>(p, acc, sums);
+  const bool solid = __syncthreads_or(acc.solid);
+  if (lane + warp * kLanes == 0) tile_record<STORE>(p, tile, x0, y0, solid, sums, partials);
 }
 
 // Consecutive steps are launched dependently (launch_pdl): once every block has

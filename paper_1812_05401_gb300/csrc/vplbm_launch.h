@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include <utility>
+
 #include "vplbm_params.h"
 
 namespace vplbm {
@@ -12,17 +14,23 @@ namespace vplbm {
 // work writes, and pdl_trigger() to let its own successor start. Behind other
 // stream work (a copy, a kernel without a trigger) it is an ordinary launch.
 template <class... Params, class... Args>
-cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, cudaStream_t st, Args&&... args) {
+cudaError_t launch_pdl_smem(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                            Args&&... args) {
   cudaLaunchAttribute attr{};
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+template <class... Params, class... Args>
+cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, cudaStream_t st, Args&&... args) {
+  return launch_pdl_smem(kernel, grid, block, 0, st, std::forward<Args>(args)...);
 }
 
 #define VPLBM_DECLARE_LAUNCHERS(SUFFIX)                                                         \
@@ -48,5 +56,10 @@ VPLBM_DECLARE_LAUNCHERS(f64)
 VPLBM_DECLARE_LAUNCHERS(f32)
 VPLBM_DECLARE_LAUNCHERS(f16)
 VPLBM_DECLARE_LAUNCHERS(bf16)
+
+// Two steps in one launch (FP32, two-rate collision, tiles of kPairRows rows);
+// prepare: once per device before the first launch.
+cudaError_t prepare_pair_f32();
+cudaError_t launch_pair_f32(const PairParams& pp, cudaStream_t st);
 
 }  // namespace vplbm

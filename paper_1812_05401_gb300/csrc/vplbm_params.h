@@ -62,6 +62,9 @@ __host__ __device__ constexpr int tile_x(int storage) { return kLanes * npt(stor
 constexpr int kNodeThreads = 256;
 constexpr int kNodeBlocks = 4;
 
+// Rows of a tile that the paired step takes at a time (vplbm_pair.cuh).
+constexpr int kPairRows = 16;
+
 // Block shape of the per-node kernels (initialisation, moments, import/export).
 constexpr int kBlockX = 64;
 constexpr int kBlockY = 4;
@@ -136,6 +139,12 @@ struct StepParams {
   int collision;            // kTrt | kMrt (read by the grouped kernel)
   int force_free;           // 1: no body force (g = 0), so fluid nodes feel no force
   unsigned round_key;       // stochastic rounding: key of the seed, mixed with the step
+};
+
+// Two consecutive steps of one launch: a.src and a.ghost_src are read,
+// b.dst and b.ghost_dst written; a.ghost_dst is null.
+struct PairParams {
+  StepParams a, b;
 };
 
 __host__ __device__ constexpr int elem_bytes(int storage) {
