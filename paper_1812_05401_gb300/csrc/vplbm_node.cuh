@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(kNodeThreads, kNodeBlocks)
   using T = typename S::T;
   using E = typename S::E;
   constexpr int N = npt(STORE), TX = tile_x(STORE), W = warps_per_block(STORE);
-  constexpr bool REF = S::kSixteen;
+  constexpr bool REF = S::kElements;
   __shared__ T s_dm[kNodeThreads], s_fx[kNodeThreads], s_fy[kNodeThreads];
   const int tile = blockIdx.x / W, w = blockIdx.x % W;
   const int tx = tile % p.tiles_x, ty = tile / p.tiles_x;
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kNodeThreads, kNodeBlocks)
         for (int a = 0; a < 9; ++a) h[a] = h[a] - sref<S>(p, a);
       }
     }
-    if (!(q.rho > T(0) && q.rho < T(1e30))) atomicOr(p.flag, 1);
+    if (!sound_density(q.rho)) atomicOr(p.flag, 1);
     drho = q.drho;
     if (m) {
       solid = true;

@@ -90,7 +90,7 @@ __device__ __forceinline__ void pair_halo(const StepParams& p, PairTile<STORE>& 
       q = macros<T, kGeneral>(p, h, m, x, y);
       collide_trt<T, kGeneral>(p, h, q);
     }
-    if (!(q.rho > T(0) && q.rho < T(1e30))) atomicOr(p.flag, 1);
+    if (!sound_density(q.rho)) atomicOr(p.flag, 1);
   }
   const T o0 = side ? h[3] : h[1], o1 = side ? h[6] : h[5], o2 = side ? h[7] : h[8];
   T(*to)[R] = sm.halo[side];
