@@ -60,6 +60,10 @@ __device__ __forceinline__ void tile_partial(const ReduceArgs& a, const double* 
   double m64 = 0.0;
   float m32 = 0.f;
   v[0] = v[1] = 0.0;
+  // four units' loads at once: one after the other they were most of a single
+  // step's sum (one monitored 1024 x 256 step with its force and field, alone,
+  // mean of three: 88.7 -> 81.2 us)
+#pragma unroll 4
   for (int w = 0; w < a.units; ++w) {
     v[0] += __ldcg(u + 3 * w + 0);
     v[1] += __ldcg(u + 3 * w + 1);
