@@ -16,7 +16,7 @@ namespace vplbm {
 //
 // A single step is bound by HBM (16384 x 4096: 0.773 ms with the mask's update,
 // 74 bytes a node); this kernel moves half the bytes and is bound by instruction
-// issue and latency at 24 warps an SM (IPC 1.75). Per step, single against pair:
+// issue and latency at 24 warps an SM (IPC 1.95). Per step, single against pair:
 // 16384 x 4096 773 -> 625 us, 4096 x 1024 51.7 -> 45.2, 6048 x 2016 (SRT,
 // convective) 150 -> 133. What it took, on 16384 x 4096 (us a step, tiles of one
 // part):
