@@ -593,6 +593,8 @@ __device__ __forceinline__ void collide_trt(const StepParams& p, T h[9], const M
 // Rates of the conserved moments (rho, j_x, j_y) do not change the result
 // (j* = j + F for any rate, because m_eq uses the half-force velocity).
 // f* = M^-1 m* with M^-1 = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4).
+// Products that are rounded, or whose fusing shows in the result, are written
+// out (mul, mad); the plain ones are by powers of two, exact either way.
 template <class T>
 __device__ __forceinline__ void collide_mrt(const StepParams& p, T h[9], const Macro<T>& q) {
   const Consts<T>& c = consts<T>(p);
@@ -609,42 +611,44 @@ __device__ __forceinline__ void collide_mrt(const StepParams& p, T h[9], const M
   const T pxy = (h[5] - h[6]) + (h[7] - h[8]);
 
   const T rho = q.rho, ux = q.ux, uy = q.uy, Fx = q.Fx, Fy = q.Fy;
-  const T uu = ux * ux + uy * uy;
-  const T uF = ux * Fx + uy * Fy;
-  const T e_eq = -T(2) * q.drho + T(3) * rho * uu;
-  const T eps_eq = q.drho - T(3) * rho * uu;
+  const T uu = mad(ux, ux, mul(uy, uy));
+  const T uF = mad(ux, Fx, mul(uy, Fy));
+  const T rho3 = mul(T(3), rho), rux = mul(rho, ux);
+  const T e_eq = mad(rho3, uu, -T(2) * q.drho);
+  const T eps_eq = mad(-rho3, uu, q.drho);
 
-  const T es = e - s1 * (e - e_eq) + (T(1) - T(0.5) * s1) * T(6) * uF;
-  const T epss = eps - s2 * (eps - eps_eq) - (T(1) - T(0.5) * s2) * T(6) * uF;
+  const T es = mad(mul(T(1) - T(0.5) * s1, T(6)), uF, mad(-s1, e - e_eq, e));
+  const T epss = mad(-mul(T(1) - T(0.5) * s2, T(6)), uF, mad(-s2, eps - eps_eq, eps));
   const T jxs = jx + Fx;
   const T jys = jy + Fy;
-  const T qxs = qx - s4 * (qx + rho * ux) - (T(1) - T(0.5) * s4) * Fx;
-  const T qys = qy - s6 * (qy + rho * uy) - (T(1) - T(0.5) * s6) * Fy;
-  const T pxxs = pxx - s7 * (pxx - rho * (ux * ux - uy * uy)) +
-                 (T(1) - T(0.5) * s7) * T(2) * (ux * Fx - uy * Fy);
-  const T pxys = pxy - s8 * (pxy - rho * ux * uy) + (T(1) - T(0.5) * s8) * (ux * Fy + uy * Fx);
+  const T qxs = mad(-(T(1) - T(0.5) * s4), Fx, mad(-s4, qx + rux, qx));
+  const T qys = mad(-(T(1) - T(0.5) * s6), Fy, mad(-s6, mad(rho, uy, qy), qy));
+  const T pxxs = mad((T(1) - T(0.5) * s7) * T(2), mad(ux, Fx, -mul(uy, Fy)),
+                     mad(-s7, mad(-rho, mad(ux, ux, -mul(uy, uy)), pxx), pxx));
+  const T pxys = mad(T(1) - T(0.5) * s8, mad(ux, Fy, mul(uy, Fx)), mad(-s8, mad(-rux, uy, pxy), pxy));
 
-  const T a0 = q.drho * T(1.0 / 9.0);
-  const T a1 = es * T(1.0 / 36.0);
-  const T a2 = epss * T(1.0 / 36.0);
-  const T a3 = jxs * T(1.0 / 6.0);
-  const T a4 = qxs * T(1.0 / 12.0);
-  const T a5 = jys * T(1.0 / 6.0);
-  const T a6 = qys * T(1.0 / 12.0);
+  const T a0 = mul(q.drho, T(1.0 / 9.0));
+  const T a1 = mul(es, T(1.0 / 36.0));
+  const T a2 = mul(epss, T(1.0 / 36.0));
+  const T a4 = mul(qxs, T(1.0 / 12.0));
+  const T a6 = mul(qys, T(1.0 / 12.0));
   const T a7 = pxxs * T(0.25);
   const T a8 = pxys * T(0.25);
+  // j*/6 - q*/6 (directions 1..4) and j*/6 + q*/12 (5..8)
+  const T x14 = mad(jxs, T(1.0 / 6.0), -T(2) * a4), x58 = mad(jxs, T(1.0 / 6.0), a4);
+  const T y14 = mad(jys, T(1.0 / 6.0), -T(2) * a6), y58 = mad(jys, T(1.0 / 6.0), a6);
 
   const T b14 = a0 - a1 - T(2) * a2;  // common part of directions 1..4
   const T b58 = a0 + T(2) * a1 + a2;  // common part of directions 5..8
   h[0] = a0 - T(4) * a1 + T(4) * a2;
-  h[1] = b14 + (a3 - T(2) * a4) + a7;
-  h[2] = b14 + (a5 - T(2) * a6) - a7;
-  h[3] = b14 - (a3 - T(2) * a4) + a7;
-  h[4] = b14 - (a5 - T(2) * a6) - a7;
-  h[5] = b58 + (a3 + a4) + (a5 + a6) + a8;
-  h[6] = b58 - (a3 + a4) + (a5 + a6) - a8;
-  h[7] = b58 - (a3 + a4) - (a5 + a6) + a8;
-  h[8] = b58 + (a3 + a4) - (a5 + a6) - a8;
+  h[1] = b14 + x14 + a7;
+  h[2] = b14 + y14 - a7;
+  h[3] = b14 - x14 + a7;
+  h[4] = b14 - y14 - a7;
+  h[5] = b58 + x58 + y58 + a8;
+  h[6] = b58 - x58 + y58 - a8;
+  h[7] = b58 - x58 - y58 + a8;
+  h[8] = b58 + x58 - y58 - a8;
 }
 
 // ---------------------------------------------------------------------------
