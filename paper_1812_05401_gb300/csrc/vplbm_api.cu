@@ -241,6 +241,7 @@ struct vplbm_solver {
 
   int64_t t = 0;
   int64_t ring_read = 0;  // first step not yet returned by vplbm_forces
+  int64_t window = 0;     // steps before t whose partials await their sum (sum_window)
   std::vector<vplbm_body> bodies;
   bool moving = false;
   bool pair = false;             // consecutive steps run two a launch (vplbm_pair.cuh)
@@ -668,6 +669,16 @@ cudaError_t launch_reduce(const ReduceArgs& a, cudaStream_t st) {
   return launch_pdl(reduce_kernel, dim3(unsigned(a.steps), reduce_chunks(a.n_tiles)), dim3(kThreads), st, a);
 }
 
+// Sums the records of the steps made since the last sum. vplbm_step leaves none
+// open unless a launch fails; every call that needs the records, their scratch
+// or the step count they belong to makes up for that first.
+cudaError_t sum_window(vplbm_solver* s) {
+  if (s->window == 0) return cudaSuccess;
+  const cudaError_t e = launch_reduce(reduce_args(s, s->t - s->window, s->window), s->stream);
+  if (e == cudaSuccess) s->window = 0;
+  return e;
+}
+
 cudaError_t launch_fused(const vplbm_solver* s, const StepParams& p) {
   const int coll = p.collision;
   if (s->nodewise) {
@@ -1071,6 +1082,7 @@ vplbm_status vplbm_set_initial_velocity(vplbm_solver* s, const double* u) {
   if ((st = init_outlet_state(s)) != VPLBM_OK) return st;
   s->t = 0;
   s->ring_read = 0;
+  s->window = 0;
   s->me_read = 0;
   s->me_stop = 0;
   VP_CUDA(s, cudaMemsetAsync(s->flag, 0, sizeof(int), s->stream));
@@ -1156,18 +1168,26 @@ vplbm_status vplbm_step(vplbm_solver* s, int64_t n) {
   if (st != VPLBM_OK) return st;
   if (n < 0) return fail(s, VPLBM_ERR_INVALID, "n must be >= 0");
   TraceRange trace("vplbm_step");
+  VP_CUDA(s, sum_window(s));
   const int most = step_window(s, n);
   if (s->sticky) return VPLBM_ERR_CUDA;
+  // a call that fails half-way (out of memory) has made its first steps: their
+  // records are summed on every way out
+  struct SumOnReturn {
+    vplbm_solver* s;
+    ~SumOnReturn() {
+      if (!s->sticky && sum_window(s) != cudaSuccess) cudaGetLastError();  // the next call tries again
+    }
+  } sum_on_return{s};
   const long long records = 3ll * s->n_tiles * (s->nodewise ? warps_per_block(s->cfg.storage) : 1);  // of a step
   // momentum exchange reads the populations of every step
   const bool pairs = s->pair && !s->me_on && (!s->moving || s->mask_next);
-  int64_t window = 0;  // steps whose partials await their sum
   for (int64_t k = 0; k < n;) {
     if ((st = ensure_mask(s, s->t)) != VPLBM_OK) return st;
     StepParams p = step_params(s, s->t, 0);
     if (s->unit_records) p.partials = s->unit_records;
-    p.partials += records * window;
-    const int count = pairs && n - k >= 2 && window + 2 <= most ? 2 : 1;
+    p.partials += records * s->window;
+    const int count = pairs && n - k >= 2 && s->window + 2 <= most ? 2 : 1;
     PairParams pp;
     if (count == 2) {
       if (s->moving && (st = ensure_next_mask(s, s->t)) != VPLBM_OK) return st;
@@ -1197,11 +1217,8 @@ vplbm_status vplbm_step(vplbm_solver* s, int64_t n) {
     s->cur ^= 1;
     s->t += count;
     k += count;
-    window += count;
-    if (window == most || k == n) {
-      VP_CUDA(s, launch_reduce(reduce_args(s, s->t - window, window), s->stream));
-      window = 0;
-    }
+    s->window += count;
+    if (s->window == most || k == n) VP_CUDA(s, sum_window(s));
   }
   return VPLBM_OK;
 }
@@ -1300,6 +1317,7 @@ vplbm_status vplbm_forces(vplbm_solver* s, double* fx, double* fy, double* mass,
   if (st != VPLBM_OK) return st;
   if (count) *count = 0;
   if (cap < 0) return fail(s, VPLBM_ERR_INVALID, "cap must be >= 0");
+  VP_CUDA(s, sum_window(s));
   const int64_t L = s->cfg.force_ring_len;
   const int64_t k = std::min(std::min(s->t - s->ring_read, L), cap);
   std::vector<double> host(3 * size_t(std::max<int64_t>(k, 1)));
@@ -1454,6 +1472,7 @@ vplbm_status vplbm_load_state(vplbm_solver* s, const void* buf, size_t bytes) {
   // pageable host-to-device copies have been staged when they return
   s->t = h.t;
   s->ring_read = h.t;
+  s->window = 0;
   s->me_read = h.t;
   s->me_stop = h.t;
   s->mask_t = s->moving ? h.t : -1;
@@ -1466,6 +1485,7 @@ vplbm_status vplbm_forces_async(vplbm_solver* s, double* records, int64_t cap, i
   if (st != VPLBM_OK) return st;
   if (count) *count = 0;
   if (cap < 0 || (cap > 0 && !records)) return fail(s, VPLBM_ERR_INVALID, "bad output buffer");
+  VP_CUDA(s, sum_window(s));
   const int64_t L = s->cfg.force_ring_len;
   const int64_t k = std::min(std::min(s->t - s->ring_read, L), cap);
   int64_t done = 0;
@@ -1557,6 +1577,7 @@ vplbm_status vplbm_set_initial_perturbation(vplbm_solver* s, double u0x, double 
   if ((st = init_outlet_state(s)) != VPLBM_OK) return st;
   s->t = 0;
   s->ring_read = 0;
+  s->window = 0;
   s->me_read = 0;
   s->me_stop = 0;
   VP_CUDA(s, cudaMemsetAsync(s->flag, 0, sizeof(int), s->stream));
@@ -1579,6 +1600,7 @@ vplbm_status vplbm_group_step(vplbm_solver* const* solvers, int32_t n, const int
     if (steps[i] < 0) return fail(s, VPLBM_ERR_INVALID, "steps must be >= 0");
     for (int j = 0; j < i; ++j)
       if (solvers[j] == s) return fail(s, VPLBM_ERR_INVALID, "a solver appears twice in the group");
+    VP_CUDA(s, sum_window(s));
     max_steps = std::max(max_steps, steps[i]);
   }
   vplbm_solver* s0 = solvers[0];

@@ -1,0 +1,90 @@
+// Drives the library's host code on the CPU (fake_cuda.h in place of the CUDA
+// runtime). One path per argument; exits 0 if it holds.
+#include "fake_cuda.h"
+
+#include "vplbm.h"
+#include "vplbm_params.h"
+
+using vplbm::ReduceArgs;
+
+#define CHECK(cond)                                                  \
+  do {                                                               \
+    if (!(cond)) {                                                   \
+      fprintf(stderr, "%s:%d: %s\n", __FILE__, __LINE__, #cond);     \
+      return 1;                                                      \
+    }                                                                \
+  } while (0)
+
+static vplbm_solver* create(int nx, int ny, int storage = VPLBM_F32) {
+  vplbm_config c;
+  vplbm_config_init(&c);
+  c.nx = nx;
+  c.ny = ny;
+  c.storage = storage;
+  c.collision = VPLBM_MRT;
+  c.tau = 0.6;
+  c.force_ring_len = 256;
+  vplbm_solver* s = nullptr;
+  if (vplbm_create(&c, &s) != VPLBM_OK) return nullptr;
+  g_launches.clear();
+  return s;
+}
+
+// (t0, steps) of each sum of records launched so far.
+static std::vector<std::pair<long long, long long>> sums() {
+  std::vector<std::pair<long long, long long>> r;
+  for (const auto& l : g_launches)
+    if (l.arg.size() == sizeof(ReduceArgs) && l.kernel.find("reduce_kernel") != std::string::npos) {
+      ReduceArgs a;
+      memcpy(&a, l.arg.data(), sizeof(a));
+      r.push_back({a.t0, a.steps});
+    }
+  return r;
+}
+using Sums = std::vector<std::pair<long long, long long>>;
+
+// A call that runs out of memory after some of its steps has still summed
+// their records.
+static int records_of_a_failed_call(int nx, int ny) {
+  vplbm_solver* s = create(nx, ny);
+  CHECK(s);
+  CHECK(vplbm_enable_timing(s, 1) == VPLBM_OK);
+  g_fail_at["cudaEventCreate"] = 5;  // two events a launch: the third launch's first
+  CHECK(vplbm_step(s, 6) == VPLBM_ERR_NOMEM);
+  const long long made = vplbm_step_count(s);
+  CHECK(made == (nx * ny > 4000000 ? 4 : 2));  // large FP32 grids: two steps a launch
+  CHECK((sums() == Sums{{0, made}}));
+  double fx[8];
+  int64_t n = 0;
+  CHECK(vplbm_forces(s, fx, nullptr, nullptr, 8, &n) == VPLBM_OK && n == made);
+  CHECK(vplbm_step(s, 3) == VPLBM_OK && vplbm_step_count(s) == made + 3);
+  CHECK((sums() == Sums{{0, made}, {made, 3}}));
+  vplbm_destroy(s);
+  return 0;
+}
+
+// The same where the sum's own launch fails: the next call makes it.
+static int records_of_a_failed_sum() {
+  vplbm_solver* s = create(300, 100);
+  CHECK(s);
+  g_fail_at["launch"] = 4;  // the third step
+  CHECK(vplbm_step(s, 1) == VPLBM_OK);
+  CHECK(vplbm_step(s, 5) == VPLBM_ERR_NOMEM && vplbm_step_count(s) == 2);
+  CHECK((sums() == Sums{{0, 1}, {1, 1}}));
+  g_fail_at["launch"] = 2;
+  CHECK(vplbm_step(s, 1) == VPLBM_ERR_NOMEM && vplbm_step_count(s) == 3);  // its sum failed, then was made
+  CHECK((sums() == Sums{{0, 1}, {1, 1}, {2, 1}}));
+  vplbm_destroy(s);
+  return 0;
+}
+
+int main(int argc, char** argv) {
+  g_keep["reduce_kernel"] = sizeof(ReduceArgs);
+  const std::string path = argc > 1 ? argv[1] : "";
+  if (path == "failed_call") return records_of_a_failed_call(300, 100);
+  if (path == "failed_call_vector") return records_of_a_failed_call(2048, 512);
+  if (path == "failed_call_pairs") return records_of_a_failed_call(2049, 2049);
+  if (path == "failed_sum") return records_of_a_failed_sum();
+  fprintf(stderr, "no such path: %s\n", path.c_str());
+  return 2;
+}
