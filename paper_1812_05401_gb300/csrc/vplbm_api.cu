@@ -863,6 +863,16 @@ size_t partials_bytes(int nt) { return 3 * sizeof(double) * size_t(kWindow) * si
 size_t chunk_sums_bytes(int nt) { return 3 * sizeof(double) * size_t(kWindow) * size_t(reduce_chunks(nt)); }
 size_t counters_bytes() { return sizeof(unsigned) * size_t(kWindow); }
 
+// Whether the solver's stream is being captured into a graph (or cannot say).
+bool capturing(const vplbm_solver* s) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s->stream, &status) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return status != cudaStreamCaptureStatusNone;
+}
+
 // Steps whose records the scratch holds. One node per thread writes several
 // record units a tile: the tiles' scratch then holds a few steps, and calls of
 // more steps take a window of units (12 bytes a node for FP32) when first made,
@@ -874,11 +884,8 @@ int step_window(vplbm_solver* s, int64_t n) {
   if (!s->nodewise) return kWindow;
   const int units = warps_per_block(s->cfg.storage);
   const int few = kWindow / units;
-  if (n > few && !s->unit_records && !s->units_refused) {
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s->stream, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone)
-      s->units_refused = mem_get(s, &s->unit_records, partials_bytes(s->n_tiles) * units) != VPLBM_OK;
-  }
+  if (n > few && !s->unit_records && !s->units_refused && !capturing(s))
+    s->units_refused = mem_get(s, &s->unit_records, partials_bytes(s->n_tiles) * units) != VPLBM_OK;
   return s->unit_records ? kWindow : few;
 }
 
@@ -1180,16 +1187,22 @@ vplbm_status vplbm_step(vplbm_solver* s, int64_t n) {
     }
   } sum_on_return{s};
   const long long records = 3ll * s->n_tiles * (s->nodewise ? warps_per_block(s->cfg.storage) : 1);  // of a step
-  // momentum exchange reads the populations of every step
-  const bool pairs = s->pair && !s->me_on && (!s->moving || s->mask_next);
+  // Pairs, then single steps. Momentum exchange reads the populations of every
+  // step. A captured call keeps an even number of pairs, so that it swaps the
+  // buffers as n single steps do: a graph of an even number of steps ends in the
+  // buffer it began with, and each replay goes on from the last one's result.
+  int64_t pairs = s->pair && !s->me_on && (!s->moving || s->mask_next) ? n / 2 : 0;
+  if (pairs > 0 && capturing(s)) pairs -= pairs % 2;
   for (int64_t k = 0; k < n;) {
     if ((st = ensure_mask(s, s->t)) != VPLBM_OK) return st;
     StepParams p = step_params(s, s->t, 0);
     if (s->unit_records) p.partials = s->unit_records;
     p.partials += records * s->window;
-    const int count = pairs && n - k >= 2 && s->window + 2 <= most ? 2 : 1;
+    static_assert(kWindow % 2 == 0, "a window is filled by pairs");
+    const int count = pairs > 0 ? 2 : 1;
     PairParams pp;
     if (count == 2) {
+      --pairs;
       if (s->moving && (st = ensure_next_mask(s, s->t)) != VPLBM_OK) return st;
       pp.a = pp.b = p;
       pp.a.ghost_dst = nullptr;  // advanced once, by the second step

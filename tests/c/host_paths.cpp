@@ -78,6 +78,25 @@ static int records_of_a_failed_sum() {
   return 0;
 }
 
+// A captured call of n steps swaps the two population buffers as often as n
+// single steps do (odd or even), and still makes n steps.
+static int captured_pairs() {
+  vplbm_solver* s = create(2049, 2049);
+  CHECK(s);
+  g_capturing = true;
+  long long t = 0;
+  for (int n = 1; n <= 9; ++n) {
+    g_launches.clear();
+    CHECK(vplbm_step(s, n) == VPLBM_OK);
+    CHECK(vplbm_step_count(s) == (t += n));
+    const int twos = launches_of("pair_step_kernel"), ones = launches_of("fused_step_kernel");
+    CHECK(2 * twos + ones == n && (twos + ones) % 2 == n % 2);
+    CHECK(twos >= n / 2 - 1);
+  }
+  vplbm_destroy(s);
+  return 0;
+}
+
 int main(int argc, char** argv) {
   g_keep["reduce_kernel"] = sizeof(ReduceArgs);
   const std::string path = argc > 1 ? argv[1] : "";
@@ -85,6 +104,7 @@ int main(int argc, char** argv) {
   if (path == "failed_call_vector") return records_of_a_failed_call(2048, 512);
   if (path == "failed_call_pairs") return records_of_a_failed_call(2049, 2049);
   if (path == "failed_sum") return records_of_a_failed_sum();
+  if (path == "captured_pairs") return captured_pairs();
   fprintf(stderr, "no such path: %s\n", path.c_str());
   return 2;
 }

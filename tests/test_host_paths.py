@@ -38,3 +38,7 @@ def _run(program, path):
 def test_failed_calls_keep_the_records_of_their_steps(program, path):
     """One node per thread, a vector of nodes per thread, and two steps a launch."""
     _run(program, path)
+
+
+def test_captured_pairs_swap_buffers_as_single_steps(program):
+    _run(program, "captured_pairs")
