@@ -236,6 +236,7 @@ struct vplbm_solver {
 
   bool nodewise = false;  // single steps run one node per thread
   bool units_refused = false;  // no memory for unit_records
+  bool next_refused = false;   // no memory for mask_next
   int tiles_x = 0, tiles_y = 0, n_tiles = 0;
   StepParams base{};  // constants; src/dst/t/bodies filled per step
 
@@ -245,7 +246,7 @@ struct vplbm_solver {
   std::vector<vplbm_body> bodies;
   bool moving = false;
   bool pair = false;             // consecutive steps run two a launch (vplbm_pair.cuh)
-  uint8_t* mask_next = nullptr;  // pair, moving bodies: the mask of a pair's second step
+  uint8_t* mask_next = nullptr;  // pair, moving bodies: the mask of a pair's second step (taken by the first pair)
   int64_t mask_next_t = -1;      // time it reflects (-1: not a copy of the mask's static layer)
   int64_t mask_t = -1;  // time the moving bodies' mask reflects (-1: none)
 
@@ -873,19 +874,26 @@ bool capturing(const vplbm_solver* s) {
   return status != cudaStreamCaptureStatusNone;
 }
 
+// A buffer that a solver can do without, taken by the first call that gains by
+// it: not while the stream is captured, where the memory would belong to the
+// graph, and not again once refused. Whether the solver has it.
+template <class T>
+bool late_get(vplbm_solver* s, T** p, size_t bytes, bool* refused) {
+  if (!*p && !*refused && !capturing(s)) *refused = mem_get(s, p, bytes) != VPLBM_OK;
+  return *p != nullptr;
+}
+
 // Steps whose records the scratch holds. One node per thread writes several
 // record units a tile: the tiles' scratch then holds a few steps, and calls of
 // more steps take a window of units (12 bytes a node for FP32) when first made,
 // so that the sums' launch (about 2 us) stays a small part of their steps
-// (1024 x 256 FP32 6.0 -> 5.2 us per step). Not while the stream captures a
-// graph, where an allocation would belong to the graph; without the memory the
-// window stays short.
+// (1024 x 256 FP32 6.0 -> 5.2 us per step). Without the memory the window stays
+// short.
 int step_window(vplbm_solver* s, int64_t n) {
   if (!s->nodewise) return kWindow;
   const int units = warps_per_block(s->cfg.storage);
   const int few = kWindow / units;
-  if (n > few && !s->unit_records && !s->units_refused && !capturing(s))
-    s->units_refused = mem_get(s, &s->unit_records, partials_bytes(s->n_tiles) * units) != VPLBM_OK;
+  if (n > few) late_get(s, &s->unit_records, partials_bytes(s->n_tiles) * units, &s->units_refused);
   return s->unit_records ? kWindow : few;
 }
 
@@ -1164,9 +1172,6 @@ vplbm_status vplbm_set_bodies(vplbm_solver* s, const vplbm_body* bodies, int32_t
   st = launch_mask_update(s, s->mask, Box{0, 0, s->cfg.nx - 1, s->cfg.ny - 1}, s->t);
   if (st != VPLBM_OK) return st;
   s->mask_t = s->moving ? s->t : -1;
-  // without memory for the second mask the steps run one a launch
-  if (s->pair && s->moving && !s->mask_next && mem_get(s, &s->mask_next, size_t(s->plane)) != VPLBM_OK && s->sticky)
-    return VPLBM_ERR_CUDA;
   return VPLBM_OK;
 }
 
@@ -1177,6 +1182,14 @@ vplbm_status vplbm_step(vplbm_solver* s, int64_t n) {
   TraceRange trace("vplbm_step");
   VP_CUDA(s, sum_window(s));
   const int most = step_window(s, n);
+  // Pairs, then single steps. Momentum exchange reads the populations of every
+  // step; moving bodies take a second mask. A captured call keeps an even number
+  // of pairs, so that it swaps the buffers as n single steps do: a graph of an
+  // even number of steps ends in the buffer it began with, and each replay goes
+  // on from the last one's result.
+  int64_t pairs = s->pair && !s->me_on ? n / 2 : 0;
+  if (pairs > 0 && s->moving && !late_get(s, &s->mask_next, size_t(s->plane), &s->next_refused)) pairs = 0;
+  if (pairs > 0 && capturing(s)) pairs -= pairs % 2;
   if (s->sticky) return VPLBM_ERR_CUDA;
   // a call that fails half-way (out of memory) has made its first steps: their
   // records are summed on every way out
@@ -1187,12 +1200,6 @@ vplbm_status vplbm_step(vplbm_solver* s, int64_t n) {
     }
   } sum_on_return{s};
   const long long records = 3ll * s->n_tiles * (s->nodewise ? warps_per_block(s->cfg.storage) : 1);  // of a step
-  // Pairs, then single steps. Momentum exchange reads the populations of every
-  // step. A captured call keeps an even number of pairs, so that it swaps the
-  // buffers as n single steps do: a graph of an even number of steps ends in the
-  // buffer it began with, and each replay goes on from the last one's result.
-  int64_t pairs = s->pair && !s->me_on && (!s->moving || s->mask_next) ? n / 2 : 0;
-  if (pairs > 0 && capturing(s)) pairs -= pairs % 2;
   for (int64_t k = 0; k < n;) {
     if ((st = ensure_mask(s, s->t)) != VPLBM_OK) return st;
     StepParams p = step_params(s, s->t, 0);

@@ -97,6 +97,37 @@ static int captured_pairs() {
   return 0;
 }
 
+// Setting bodies takes no memory, captured or not; the second mask of moving
+// bodies is taken by the first call that pairs its steps outside capture.
+static int second_mask(bool refuse) {
+  vplbm_solver* s = create(2049, 2049);
+  CHECK(s);
+  vplbm_body b{};
+  b.cx = b.cy = 1000.0;
+  b.radius = 50.0;
+  b.amp_y = 4.0;
+  b.period = 100.0;
+  const size_t allocs = g_allocs.size();
+  for (bool captured : {true, false}) {
+    g_capturing = captured;
+    CHECK(vplbm_set_bodies(s, &b, 1) == VPLBM_OK && vplbm_step(s, 1) == VPLBM_OK && g_allocs.size() == allocs);
+  }
+  g_capturing = true;
+  g_launches.clear();
+  CHECK(vplbm_step(s, 4) == VPLBM_OK && g_allocs.size() == allocs);
+  CHECK(launches_of("pair_step_kernel") == 0 && launches_of("fused_step_kernel") == 4);
+  g_capturing = false;
+  if (refuse) g_fail_at["cudaMallocAsync"] = 1;
+  for (int call = 0; call < 2; ++call) {
+    g_launches.clear();
+    CHECK(vplbm_step(s, 4) == VPLBM_OK && g_allocs.size() == allocs + (refuse ? 0 : 1));
+    CHECK(launches_of("pair_step_kernel") == (refuse ? 0 : 2) && launches_of("fused_step_kernel") == (refuse ? 4 : 0));
+  }
+  if (!refuse) CHECK(g_allocs.back() == size_t(2049) * 2080);  // a byte a node of padded rows
+  vplbm_destroy(s);
+  return 0;
+}
+
 int main(int argc, char** argv) {
   g_keep["reduce_kernel"] = sizeof(ReduceArgs);
   const std::string path = argc > 1 ? argv[1] : "";
@@ -105,6 +136,8 @@ int main(int argc, char** argv) {
   if (path == "failed_call_pairs") return records_of_a_failed_call(2049, 2049);
   if (path == "failed_sum") return records_of_a_failed_sum();
   if (path == "captured_pairs") return captured_pairs();
+  if (path == "second_mask") return second_mask(false);
+  if (path == "second_mask_refused") return second_mask(true);
   fprintf(stderr, "no such path: %s\n", path.c_str());
   return 2;
 }

@@ -42,3 +42,8 @@ def test_failed_calls_keep_the_records_of_their_steps(program, path):
 
 def test_captured_pairs_swap_buffers_as_single_steps(program):
     _run(program, "captured_pairs")
+
+
+@pytest.mark.parametrize("path", ["second_mask", "second_mask_refused"])
+def test_second_mask_is_taken_by_the_first_pair(program, path):
+    _run(program, path)
