@@ -876,10 +876,15 @@ bool capturing(const vplbm_solver* s) {
 
 // A buffer that a solver can do without, taken by the first call that gains by
 // it: not while the stream is captured, where the memory would belong to the
-// graph, and not again once refused. Whether the solver has it.
+// graph, and not again once refused. A refusal is no error of the call: the last
+// error stays as it was. Whether the solver has it.
 template <class T>
 bool late_get(vplbm_solver* s, T** p, size_t bytes, bool* refused) {
-  if (!*p && !*refused && !capturing(s)) *refused = mem_get(s, p, bytes) != VPLBM_OK;
+  if (!*p && !*refused && !capturing(s)) {
+    const std::string before = s->err;
+    *refused = mem_get(s, p, bytes) != VPLBM_OK;
+    if (*refused && !s->sticky) s->err = before;
+  }
   return *p != nullptr;
 }
 

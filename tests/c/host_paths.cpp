@@ -128,6 +128,26 @@ static int second_mask(bool refuse) {
   return 0;
 }
 
+// A buffer that a call does without leaves no error behind.
+static int refused_buffers_are_no_error(int nx, int ny, bool moving) {
+  vplbm_solver* s = create(nx, ny);
+  CHECK(s);
+  vplbm_body b{};
+  b.radius = 5.0;
+  b.amp_y = 4.0;
+  b.period = moving ? 100.0 : 0.0;
+  CHECK(vplbm_set_bodies(s, &b, 1) == VPLBM_OK);
+  for (const char* before : {"", "n must be >= 0"}) {
+    if (*before) CHECK(vplbm_step(s, -1) == VPLBM_ERR_INVALID);
+    g_fail_at["cudaMallocAsync"] = 1;
+    CHECK(vplbm_step(s, 40) == VPLBM_OK);
+    CHECK(*before || g_fail_at["cudaMallocAsync"] == 0);  // asked for, once
+    CHECK(strcmp(vplbm_last_error(s), before) == 0);
+  }
+  vplbm_destroy(s);
+  return 0;
+}
+
 int main(int argc, char** argv) {
   g_keep["reduce_kernel"] = sizeof(ReduceArgs);
   const std::string path = argc > 1 ? argv[1] : "";
@@ -138,6 +158,8 @@ int main(int argc, char** argv) {
   if (path == "captured_pairs") return captured_pairs();
   if (path == "second_mask") return second_mask(false);
   if (path == "second_mask_refused") return second_mask(true);
+  if (path == "refused_window") return refused_buffers_are_no_error(300, 100, false);
+  if (path == "refused_mask") return refused_buffers_are_no_error(2049, 2049, true);
   fprintf(stderr, "no such path: %s\n", path.c_str());
   return 2;
 }

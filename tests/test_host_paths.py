@@ -47,3 +47,8 @@ def test_captured_pairs_swap_buffers_as_single_steps(program):
 @pytest.mark.parametrize("path", ["second_mask", "second_mask_refused"])
 def test_second_mask_is_taken_by_the_first_pair(program, path):
     _run(program, path)
+
+
+@pytest.mark.parametrize("path", ["refused_window", "refused_mask"])
+def test_refused_buffers_leave_no_error(program, path):
+    _run(program, path)
