@@ -185,10 +185,10 @@ double vplbm_tau_from_reynolds(double u_ref, double l_ref, double re);
 /* Device bytes a solver with this configuration allocates at creation
  * (admission). Buffers taken later come on top when used: the static
  * solid-velocity field, the momentum-exchange records, the staging buffers
- * of host transfers, on small grids, with a call of many steps, the
- * records of up to 64 of them (12 bytes a node for FP32), and, with the first
- * call whose steps run in pairs, a second mask for moving bodies (1 byte a
- * node). 0 for an invalid configuration. */
+ * of host transfers; on small grids, with a call of many steps, the records
+ * of up to 64 of them (12 bytes a node for FP32, 8 MiB at most); with the
+ * first call whose steps run in pairs, a second mask for moving bodies (1
+ * byte a node). 0 for an invalid configuration. */
 size_t vplbm_footprint_bytes(const vplbm_config* cfg);
 
 /* Allocates the solver and sets the store to f*(0) = f_eq(rho0, u0) with an

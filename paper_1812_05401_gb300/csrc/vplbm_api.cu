@@ -213,7 +213,7 @@ struct vplbm_solver {
   uint8_t* mask = nullptr;
   void* us = nullptr;
   double* partials = nullptr;    // [kWindow][n_tiles][3], or as many steps of record units (nodewise)
-  double* unit_records = nullptr;  // nodewise, longer calls: [kWindow][n_tiles][units][3]
+  double* unit_records = nullptr;  // nodewise, longer calls: [step_window][n_tiles][units][3]
   double* chunk_sums = nullptr;  // [kWindow][n_chunks][3]
   unsigned* counters = nullptr;  // [kWindow]
   double* ring = nullptr;
@@ -892,14 +892,21 @@ bool late_get(vplbm_solver* s, T** p, size_t bytes, bool* refused) {
 // record units a tile: the tiles' scratch then holds a few steps, and calls of
 // more steps take a window of units (12 bytes a node for FP32) when first made,
 // so that the sums' launch (about 2 us) stays a small part of their steps
-// (1024 x 256 FP32 6.0 -> 5.2 us per step). Without the memory the window stays
-// short.
+// (1024 x 256 FP32 6.0 -> 5.2 us per step). The window is bounded, since it
+// comes on top of the footprint a solver is admitted by: 64 steps up to about
+// 700,000 FP32 or 350,000 FP64 nodes; larger FP64 grids, whose steps take 70 us
+// and more, get fewer or none (2 us in 8 steps). Without the memory the window
+// stays short.
+constexpr size_t kUnitRecordBytes = size_t(8) << 20;
 int step_window(vplbm_solver* s, int64_t n) {
   if (!s->nodewise) return kWindow;
   const int units = warps_per_block(s->cfg.storage);
   const int few = kWindow / units;
-  if (n > few) late_get(s, &s->unit_records, partials_bytes(s->n_tiles) * units, &s->units_refused);
-  return s->unit_records ? kWindow : few;
+  const size_t step_bytes = 3 * sizeof(double) * size_t(s->n_tiles) * units;
+  const int most = int(std::min<size_t>(kWindow, kUnitRecordBytes / step_bytes));
+  if (most < 2 * few) return few;
+  if (n > few) late_get(s, &s->unit_records, step_bytes * most, &s->units_refused);
+  return s->unit_records ? most : few;
 }
 
 vplbm_status check_usable(vplbm_solver* s) {

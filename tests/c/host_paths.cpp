@@ -2,6 +2,8 @@
 // runtime). One path per argument; exits 0 if it holds.
 #include "fake_cuda.h"
 
+#include <algorithm>
+
 #include "vplbm.h"
 #include "vplbm_params.h"
 
@@ -148,6 +150,32 @@ static int refused_buffers_are_no_error(int nx, int ny, bool moving) {
   return 0;
 }
 
+// Stepping takes at most 8 MiB beyond what creation took, whatever the grid,
+// and no window of records is longer than what was taken (a tile's scratch at
+// creation holds 64 partials, eight steps of eight units).
+static int bounded_window(int nx, int ny, int storage) {
+  vplbm_solver* s = create(nx, ny, storage);
+  CHECK(s);
+  const size_t allocs = g_allocs.size();
+  for (int n : {1, 8, 200, 9}) CHECK(vplbm_step(s, n) == VPLBM_OK);
+  size_t late = 0;
+  for (size_t i = allocs; i < g_allocs.size(); ++i) late += g_allocs[i];
+  CHECK(late <= size_t(8) << 20);
+  long long t = 0;
+  for (const auto& l : g_launches) {
+    if (l.arg.empty()) continue;
+    ReduceArgs a;
+    memcpy(&a, l.arg.data(), sizeof(a));
+    CHECK(a.t0 == t);
+    t += a.steps;
+    const size_t bytes = size_t(a.steps) * a.n_tiles * (a.units ? a.units : 1) * 24;
+    CHECK(bytes <= std::max(late, size_t(a.n_tiles) * 64 * 24));
+  }
+  CHECK(t == 218);
+  vplbm_destroy(s);
+  return 0;
+}
+
 int main(int argc, char** argv) {
   g_keep["reduce_kernel"] = sizeof(ReduceArgs);
   const std::string path = argc > 1 ? argv[1] : "";
@@ -160,6 +188,10 @@ int main(int argc, char** argv) {
   if (path == "second_mask_refused") return second_mask(true);
   if (path == "refused_window") return refused_buffers_are_no_error(300, 100, false);
   if (path == "refused_mask") return refused_buffers_are_no_error(2049, 2049, true);
+  if (path == "window_f64") return bounded_window(2048, 1024, VPLBM_F64);
+  if (path == "window_f64_mid") return bounded_window(1024, 512, VPLBM_F64);
+  if (path == "window_f32") return bounded_window(700, 700, VPLBM_F32);
+  if (path == "window_f16") return bounded_window(128, 64, VPLBM_F16_OFFSET);
   fprintf(stderr, "no such path: %s\n", path.c_str());
   return 2;
 }

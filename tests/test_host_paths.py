@@ -52,3 +52,8 @@ def test_second_mask_is_taken_by_the_first_pair(program, path):
 @pytest.mark.parametrize("path", ["refused_window", "refused_mask"])
 def test_refused_buffers_leave_no_error(program, path):
     _run(program, path)
+
+
+@pytest.mark.parametrize("path", ["window_f64", "window_f64_mid", "window_f32", "window_f16"])
+def test_record_windows_are_bounded(program, path):
+    _run(program, path)
