@@ -176,6 +176,30 @@ static int bounded_window(int nx, int ny, int storage) {
   return 0;
 }
 
+// A grouped call takes one buffer and makes one copy for its tables, whatever
+// the storages and schemes of its solvers.
+static int grouped_tables() {
+  vplbm_config c;
+  vplbm_config_init(&c);
+  c.tau = 0.6;
+  c.stream = reinterpret_cast<void*>(8);
+  vplbm_solver* s[3];
+  int64_t steps[3] = {3, 1, 2};
+  for (int i = 0; i < 3; ++i) {
+    c.nx = 300 + i;
+    c.ny = 70;
+    c.storage = i == 0 ? VPLBM_F16_OFFSET : VPLBM_F32;
+    c.streaming = i == 2 ? VPLBM_STREAM_AA : VPLBM_STREAM_AB;
+    CHECK(vplbm_create(&c, &s[i]) == VPLBM_OK);
+  }
+  g_calls.clear();
+  CHECK(vplbm_group_step(s, 3, steps) == VPLBM_OK);
+  CHECK(g_calls["cudaMallocAsync"] == 1 && g_calls["cudaMemcpyAsync"] == 1);
+  for (int i = 0; i < 3; ++i) CHECK(vplbm_step_count(s[i]) == steps[i]);
+  for (vplbm_solver* v : s) vplbm_destroy(v);
+  return 0;
+}
+
 int main(int argc, char** argv) {
   g_keep["reduce_kernel"] = sizeof(ReduceArgs);
   const std::string path = argc > 1 ? argv[1] : "";
@@ -192,6 +216,7 @@ int main(int argc, char** argv) {
   if (path == "window_f64_mid") return bounded_window(1024, 512, VPLBM_F64);
   if (path == "window_f32") return bounded_window(700, 700, VPLBM_F32);
   if (path == "window_f16") return bounded_window(128, 64, VPLBM_F16_OFFSET);
+  if (path == "grouped_tables") return grouped_tables();
   fprintf(stderr, "no such path: %s\n", path.c_str());
   return 2;
 }

@@ -57,3 +57,7 @@ def test_refused_buffers_leave_no_error(program, path):
 @pytest.mark.parametrize("path", ["window_f64", "window_f64_mid", "window_f32", "window_f16"])
 def test_record_windows_are_bounded(program, path):
     _run(program, path)
+
+
+def test_grouped_calls_copy_their_tables_at_once(program):
+    _run(program, "grouped_tables")
