@@ -213,7 +213,7 @@ struct vplbm_solver {
   uint8_t* mask = nullptr;
   void* us = nullptr;
   double* partials = nullptr;    // [kWindow][n_tiles][3], or as many steps of record units (nodewise)
-  double* unit_records = nullptr;  // nodewise, longer calls: [step_window][n_tiles][units][3]
+  double* unit_records = nullptr;  // nodewise, longer calls: [step_window][units][3][n_tiles]
   double* chunk_sums = nullptr;  // [kWindow][n_chunks][3]
   unsigned* counters = nullptr;  // [kWindow]
   double* ring = nullptr;

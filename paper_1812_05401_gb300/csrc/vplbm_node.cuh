@@ -194,10 +194,10 @@ __global__ void __launch_bounds__(kNodeThreads, kNodeBlocks)
     bfy = warp_sum(double(fy));
   }
   if (threadIdx.x == 0) {
-    double* out = p.partials + 3ll * blockIdx.x;
+    double* out = p.partials + 3ll * p.n_tiles * w + tile;
     out[0] = bfx;
-    out[1] = bfy;
-    out[2] = double(dm);
+    out[p.n_tiles] = bfy;
+    *reinterpret_cast<T*>(out + 2ll * p.n_tiles) = dm;
   }
 }
 

@@ -130,7 +130,7 @@ struct StepParams {
   Consts<double> cd;        // constants for the FP64 kernels
   Consts<float> cf;         // the same, rounded, for the FP32 kernels
   // [n_tiles][3] of this step (grouped: [kWindow][n_tiles][3]; one node per
-  // thread: [n_tiles][warps_per_block][3], the tile's record units)
+  // thread: [warps_per_block][3][n_tiles], the tiles' record units)
   double* partials;
   int* flag;                // set to 1 on divergence
   long long t;              // index of this step
@@ -170,8 +170,9 @@ struct ReduceArgs {
   long long steps;         // steps of the window (grouped: of the member's whole call)
   int n_tiles, ring_len, reduce_mass;
   // 0: a partial per tile. Otherwise the partials are per record unit (this
-  // many a tile, rows of the tile by warp) and the tile's sum is formed here,
-  // as the vector kernel forms it: densities in FP32 or (f64) FP64
+  // many a tile, rows of the tile by warp: [steps][units][3][n_tiles]) and the
+  // tile's sum is formed here, as the vector kernel forms it: densities (the
+  // third component) are FP32 or (f64) FP64 numbers, in eight bytes each
   int units, f64;
   int nx, ny, tile_x, tile_y, tiles_x;
 };

@@ -40,38 +40,50 @@ __device__ __forceinline__ void block_sum3(double v[3], double (*sm)[3]) {
     sm[warp][2] = v[2];
   }
   __syncthreads();
-  if (tid == 0) {
-    for (int k = 0; k < 3; ++k) {
-      double s = 0.0;
-      for (int w = 0; w < n_warps; ++w) s += sm[w][k];
-      v[k] = s;
-    }
+  if (warp == 0) {  // a component a lane
+    double s = 0.0;
+    for (int w = 0; w < n_warps; ++w) s += sm[w][lane % 3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v[k] = __shfl_sync(0xffffffffu, s, k);
   }
   __syncthreads();
 }
 
-// Tile i's partial of a step.
+// Tile i's partial of a step. Record units lie by unit and component, tile after
+// tile, so that the threads' loads are contiguous (a tile's units one after the
+// other cost four times the sectors, through one SM); a unit's density is an FP32
+// number where the collision is, so that it is not converted back and forth on
+// the FP64 pipe. A single step's sum is a chain of latencies that nothing hides:
+// with this, and a component a lane in block_sum3's last sum, one 1024 x 256 FP32
+// step with its record, alone, went from 22.1 to 20.5 us (three runs of each,
+// apart by 0.4 and 0.8), the sum itself from 8.5 to 7.9. Leaving out the additions of
+// zero forces by votes made it longer (8.2; 10.8 against 9.3 on 4096 x 1024).
 __device__ __forceinline__ void tile_partial(const ReduceArgs& a, const double* src, int i, double v[3]) {
   if (!a.units) {
     for (int k = 0; k < 3; ++k) v[k] = __ldcg(src + 3ll * i + k);
     return;
   }
-  const double* u = src + 3ll * i * a.units;
   double m64 = 0.0;
   float m32 = 0.f;
   v[0] = v[1] = 0.0;
-  // four units' loads at once: one after the other they were most of a single
-  // step's sum (one monitored 1024 x 256 step with its force and field, alone,
-  // mean of three: 88.7 -> 81.2 us)
-#pragma unroll 4
-  for (int w = 0; w < a.units; ++w) {
-    v[0] += __ldcg(u + 3 * w + 0);
-    v[1] += __ldcg(u + 3 * w + 1);
-    const double m = __ldcg(u + 3 * w + 2);
-    if (a.f64)
-      m64 += m;
-    else
-      m32 += float(m);
+  const long long nt = a.n_tiles;
+  constexpr int kBatch = 4;  // units whose loads are under way at once (a tile has 4 or 8)
+  for (int w0 = 0; w0 < a.units; w0 += kBatch) {
+    double x[kBatch][3];
+#pragma unroll
+    for (int w = 0; w < kBatch; ++w) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) x[w][k] = __ldcg(src + nt * (3 * (w0 + w) + k) + i);
+    }
+#pragma unroll
+    for (int w = 0; w < kBatch; ++w) {
+      v[0] += x[w][0];
+      v[1] += x[w][1];
+      if (a.f64)
+        m64 += x[w][2];
+      else
+        m32 += __int_as_float(__double2loint(x[w][2]));
+    }
   }
   const int x0 = i % a.tiles_x * a.tile_x, y0 = i / a.tiles_x * a.tile_y;
   // sum rho = active nodes + sum drho
