@@ -36,12 +36,11 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 CPU_WARMUP, CPU_STEPS = 5, 20  # the cpu_baseline leg's oracle sample (full grid)
-# FP32 A/B grids of more nodes run consecutive steps two a launch (vplbm_step)
-PAIR_NODES = 4_000_000
 ALGO_BYTES = {"f32": 73.0, "f16": 37.0, "bf16": 37.0, "f64": 145.0}  # per node update, u8 mask
 FALLBACK_HBM_GBS = 6800.0
-KERNEL_SOURCES = ["paper_1812_05401_gb300/csrc/vplbm_device.cuh", "paper_1812_05401_gb300/csrc/vplbm_params.h",
-                  "paper_1812_05401_gb300/csrc/vplbm_kernels_impl.cuh"]
+KERNEL_SOURCES = ["paper_1812_05401_gb300/csrc/" + f for f in (
+    "vplbm_device.cuh", "vplbm_params.h", "vplbm_kernels_impl.cuh", "vplbm_node.cuh", "vplbm_pair.cuh",
+    "vplbm_reduce.cuh")]
 
 
 def _code_only(text: str) -> str:
@@ -54,7 +53,7 @@ def _code_only(text: str) -> str:
 
 
 def kernel_hash() -> str:
-    """Identifies the fused kernel's code (its comments aside); DRAM counters
+    """Identifies the step kernels' code (its comments aside); DRAM counters
     taken on another code are not reported as this kernel's traffic."""
     h = hashlib.sha256()
     for f in KERNEL_SOURCES:
@@ -289,7 +288,8 @@ def workload_config(w, storage: str, streaming: str, world: int, l2_note: str | 
     return {"workload": w.name + f" {w.collision.upper()} {storage.upper()}",
             "nx": w.nx, "ny": w.ny, "nodes": w.nx * w.ny, "storage": storage,
             "collision": w.collision, "re": w.re, "u_in": w.u_ref,
-            "step": "mask update of the moving body + fused pull/penalize/collide/reduce kernel",
+            "step": "mask update of the moving body + fused pull/penalize/collide kernel (FP32 A/B: two steps a "
+                    "launch) and the sums of the step records, one launch per 64 steps",
             "streaming": streaming,
             **({"l2": l2_note} if l2_note else {}),
             "parallelism": f"replicas x{world}"}
@@ -357,6 +357,7 @@ def run_gpu(args):
             V.vplbm_enable_timing(s.h, False)
             return ms, launches, clk, fused_ms, fused_n
 
+        step_kernel = V.vplbm_step_kernel(s.h)
         ms, launches, clk, fused_ms, fused_n = timed_region()
         why = clocks_rejected(clk)
         if max_over_ranks(1.0 if why else 0.0) > 0:  # every rank re-measures, once
@@ -452,12 +453,12 @@ def run_gpu(args):
     l2_bytes = device_l2_bytes()
     resident, l2_note = l2_residency(nodes, args.storage, args.streaming, l2_bytes)
     kms = fused_ms / max(fused_n, 1)
-    # large FP32 A/B grids run two steps a launch, which read and write the
-    # populations once (fused_n counts steps: kms is the time of one)
-    paired = args.storage == "f32" and args.streaming == "ab" and nodes > PAIR_NODES and args.steps > 1
+    # two steps a launch read and write the populations once (fused_n counts
+    # steps: kms is the time of one; traffic is that of a launch)
+    paired = step_kernel == "pair_step_kernel" and args.steps > 1
     algo = ALGO_BYTES[args.storage] - (36 if paired else 0)
     achieved = algo * nodes / (kms / 1e3) / 1e9
-    traffic = None if paired else traffic_per_launch(args.workload, args.storage, args.streaming)
+    traffic = traffic_per_launch(args.workload, args.storage, args.streaming)
     result = {
         "metric": "VP-LBM MLUPS (node updates per second / 1e6)",
         "value": round(value, 1),
@@ -479,7 +480,7 @@ def run_gpu(args):
                      "frac": round(achieved / peak, 4), "traffic": traffic,
                      "peak_source": f"{peak_src} copy bandwidth",
                      "kernel": "pair_step_kernel<F32> (per step, two steps a launch)" if paired else
-                     f"fused_step_kernel<{args.storage.upper()},{w.collision.upper()}>" + (
+                     f"{step_kernel}<{args.storage.upper()},{w.collision.upper()}>" + (
                          "" if args.streaming == "ab" else " (in place: push and local steps)"),
                      "kernel_ms": round(kms, 4), "algo_bytes_per_node": algo,
                      "algo_bytes_per_launch": algo * nodes * (2 if paired else 1),

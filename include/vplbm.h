@@ -322,9 +322,14 @@ vplbm_status vplbm_group_step(vplbm_solver* const* solvers, int32_t n,
                               const int64_t* steps);
 
 /* Kernel launches this solver issued on its hot path (fused steps, one launch
- * for two where they run in pairs, and mask updates; the sums of step records, one per up to 64 steps of a call, are not
- * counted) since creation. */
+ * for two where they run in pairs, and mask updates; the sums of step records,
+ * one per up to 64 steps of a call, are not counted) since creation. */
 int64_t vplbm_launch_count(const vplbm_solver* s);
+
+/* Name of the kernel that a call of several steps of this solver runs now:
+ * "pair_step_kernel" (two steps a launch), "node_step_kernel" (one node per
+ * thread) or "fused_step_kernel". NULL for a NULL handle. */
+const char* vplbm_step_kernel(const vplbm_solver* s);
 
 /* Timing of the fused step kernel: enable = 1 brackets each fused launch with
  * CUDA events on the solver's stream. vplbm_fused_timing synchronizes and

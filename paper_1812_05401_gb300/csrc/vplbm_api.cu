@@ -888,6 +888,10 @@ bool late_get(vplbm_solver* s, T** p, size_t bytes, bool* refused) {
   return *p != nullptr;
 }
 
+// Whether the solver's steps run in pairs now: momentum exchange reads the
+// populations of every step. (Moving bodies take a second mask as well.)
+bool steps_pair(const vplbm_solver* s) { return s->pair && !s->me_on; }
+
 // Steps whose records the scratch holds. One node per thread writes several
 // record units a tile: the tiles' scratch then holds a few steps, and calls of
 // more steps take a window of units (12 bytes a node for FP32) when first made,
@@ -1194,12 +1198,11 @@ vplbm_status vplbm_step(vplbm_solver* s, int64_t n) {
   TraceRange trace("vplbm_step");
   VP_CUDA(s, sum_window(s));
   const int most = step_window(s, n);
-  // Pairs, then single steps. Momentum exchange reads the populations of every
-  // step; moving bodies take a second mask. A captured call keeps an even number
-  // of pairs, so that it swaps the buffers as n single steps do: a graph of an
-  // even number of steps ends in the buffer it began with, and each replay goes
-  // on from the last one's result.
-  int64_t pairs = s->pair && !s->me_on ? n / 2 : 0;
+  // Pairs, then single steps. A captured call keeps an even number of pairs, so
+  // that it swaps the buffers as n single steps do: a graph of an even number of
+  // steps ends in the buffer it began with, and each replay goes on from the last
+  // one's result.
+  int64_t pairs = steps_pair(s) ? n / 2 : 0;
   if (pairs > 0 && s->moving && !late_get(s, &s->mask_next, size_t(s->plane), &s->next_refused)) pairs = 0;
   if (pairs > 0 && capturing(s)) pairs -= pairs % 2;
   if (s->sticky) return VPLBM_ERR_CUDA;
@@ -1757,6 +1760,12 @@ vplbm_status vplbm_group_step(vplbm_solver* const* solvers, int32_t n, const int
 }
 
 int64_t vplbm_launch_count(const vplbm_solver* s) { return s ? s->launches : -1; }
+
+const char* vplbm_step_kernel(const vplbm_solver* s) {
+  if (!s) return nullptr;
+  if (steps_pair(s) && !(s->moving && s->next_refused)) return "pair_step_kernel";
+  return s->nodewise ? "node_step_kernel" : "fused_step_kernel";
+}
 
 vplbm_status vplbm_enable_timing(vplbm_solver* s, int32_t enable) {
   vplbm_status st = check_usable(s);

@@ -111,6 +111,8 @@ def lib() -> C.CDLL:
         L.vplbm_group_step.argtypes = [C.POINTER(P), C.c_int32, C.POINTER(C.c_int64)]
         L.vplbm_launch_count.argtypes = [P]
         L.vplbm_launch_count.restype = C.c_int64
+        L.vplbm_step_kernel.argtypes = [P]
+        L.vplbm_step_kernel.restype = C.c_char_p
         L.vplbm_enable_timing.argtypes = [P, C.c_int32]
         L.vplbm_fused_timing.argtypes = [P, dp, C.POINTER(C.c_int64)]
         L.vplbm_last_error.argtypes = [P]
@@ -354,6 +356,10 @@ def vplbm_group_step(handles, steps):
 
 def vplbm_launch_count(h) -> int:
     return int(lib().vplbm_launch_count(h))
+
+
+def vplbm_step_kernel(h) -> str:
+    return lib().vplbm_step_kernel(h).decode()
 
 
 def vplbm_enable_timing(h, enable: bool = True):

@@ -200,6 +200,31 @@ static int grouped_tables() {
   return 0;
 }
 
+// The name of the step kernel is that of the launches a call makes.
+static int named_kernel() {
+  for (int storage : {VPLBM_F64, VPLBM_F32, VPLBM_F16_OFFSET})
+    for (int nx : {300, 1200, 2049})
+      for (int rows : {0, 8, 32})
+        for (bool exchange : {false, true}) {
+          vplbm_config c;
+          vplbm_config_init(&c);
+          c.nx = nx;
+          c.ny = nx;
+          c.tau = 0.6;
+          c.storage = storage;
+          c.tile_rows = rows;
+          vplbm_solver* s = nullptr;
+          CHECK(vplbm_create(&c, &s) == VPLBM_OK);
+          CHECK(vplbm_enable_momentum_exchange(s, exchange) == VPLBM_OK);
+          g_launches.clear();
+          CHECK(vplbm_step(s, 2) == VPLBM_OK);
+          CHECK(launches_of(vplbm_step_kernel(s)) == (strcmp(vplbm_step_kernel(s), "pair_step_kernel") ? 2 : 1));
+          CHECK(launches_of("_step_kernel") == launches_of(vplbm_step_kernel(s)));
+          vplbm_destroy(s);
+        }
+  return 0;
+}
+
 int main(int argc, char** argv) {
   g_keep["reduce_kernel"] = sizeof(ReduceArgs);
   const std::string path = argc > 1 ? argv[1] : "";
@@ -217,6 +242,7 @@ int main(int argc, char** argv) {
   if (path == "window_f32") return bounded_window(700, 700, VPLBM_F32);
   if (path == "window_f16") return bounded_window(128, 64, VPLBM_F16_OFFSET);
   if (path == "grouped_tables") return grouped_tables();
+  if (path == "named_kernel") return named_kernel();
   fprintf(stderr, "no such path: %s\n", path.c_str());
   return 2;
 }

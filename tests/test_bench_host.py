@@ -117,3 +117,17 @@ def test_clock_records_that_disqualify_a_run():
 def test_workloads_are_the_configurations_and_take_the_storage(name, nx, ny, collision):
     w = bench.make_workload(name, "bf16")
     assert (w.nx, w.ny, w.collision, w.storage) == (nx, ny, collision, "bf16")
+
+
+def test_kernel_hash_covers_every_header_of_the_step_kernels():
+    """The sources the kernels' translation units include, one from another."""
+    import re
+    csrc = os.path.join(ROOT, "paper_1812_05401_gb300", "csrc")
+    seen, todo = set(), [f for f in os.listdir(csrc) if f.startswith("kernels_")]
+    while todo:
+        for f in re.findall(r'#include "([^"]+)"', open(os.path.join(csrc, todo.pop())).read()):
+            if f not in seen:
+                seen.add(f)
+                todo.append(f)
+    seen.discard("vplbm_launch.h")  # launchers' declarations
+    assert seen == {os.path.basename(f) for f in bench.KERNEL_SOURCES}

@@ -61,3 +61,7 @@ def test_record_windows_are_bounded(program, path):
 
 def test_grouped_calls_copy_their_tables_at_once(program):
     _run(program, "grouped_tables")
+
+
+def test_the_step_kernel_has_its_name(program):
+    _run(program, "named_kernel")
