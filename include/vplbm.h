@@ -225,8 +225,9 @@ vplbm_status vplbm_set_bodies(vplbm_solver* s, const vplbm_body* bodies, int32_t
 
 /* Advances n >= 0 time steps (asynchronous). Step t maps f*(t) to f*(t+1)
  * with the mask and solid velocity of time t. On FP32 A/B grids of more than
- * 4,000,000 nodes (SRT or two-rate MRT, no momentum exchange) consecutive
- * steps of a call run two a launch, with the results of single steps. A call
+ * 4,000,000 nodes (SRT or two-rate MRT, tiles of 16 or 32 rows, no momentum
+ * exchange) consecutive steps of a call run two a launch, with the results of
+ * single steps. A call
  * captured into a graph swaps the population buffers once per step or once per
  * two, but always an odd number of times for odd n and an even one for even n:
  * a graph of an even number of steps of a flow without moving bodies can be

@@ -827,10 +827,17 @@ int tile_rows_of(const vplbm_config* c) {
 }
 
 // Whether a solver's consecutive steps run two a launch (vplbm_pair.cuh): FP32
-// grids whose populations exceed L2 (2 x 144 MB at the line). Per step, single
-// against paired: 2896 x 1448 49.6 / 45.8 us, 4096 x 1024 51.7 / 45.2, 6048 x
-// 2016 150 / 133, 16384 x 4096 773 / 625; below, L2 holds much of what a pair
-// saves: 2048 x 1024 25.8 / 26.3, 1001 x 1401 18.6 / 22.0.
+// grids whose populations exceed L2 (2 x 144 MB at the line; below, L2 holds what
+// a pair saves, and up to 3.7 million nodes tiles are 8 rows high). Per step of
+// batches of 64 in a channel with a cylinder, single against paired, tiles of the
+// automatic height in both, least of seven, three runs apart by 0.3%:
+// 2896 x 1448 49.9 / 47.7 us, 4096 x 1024 49.4 / 43.1, 3000 x 1600 55.9 / 53.6,
+// 3000 x 2000 69.8 / 65.9, 4096 x 2048 97.0 / 82.2, 6048 x 2016 (SRT, convective)
+// 142 / 126, 16384 x 4096 734 / 578; just below the line 2000 x 1990 48.2 / 48.3.
+// With a body force through 15% of solids 4096 x 1024 74.8 / 70.7, 3000 x 2000
+// 102.9 / 99.2. The line does not see everything: a last column of tiles with one
+// node (2049 x 2049 49.5 / 51.5) and forced flows in tiles of 32 rows (8000 x
+// 2000 235 / 242) lose by it.
 constexpr long long kPairNodes = 4000000;
 bool pair_rule(const vplbm_config* c) {
   StepParams consts{};
@@ -848,9 +855,14 @@ void tiles_of(const vplbm_config* c, int* tx, int* ty, int* nt) {
 }
 
 // Whether the solver's own steps run one node per thread (vplbm_node.cuh):
-// grids up to the size where the vector kernel catches up (measured there;
-// FP64 gains at every size, but a window of its record units takes 6 to 24
-// bytes a node, so larger grids keep a partial per tile).
+// grids up to the size where the vector kernel catches up. us per step, vector /
+// node kernel, channel: FP32 640 x 640 7.5 / 7.0, 700 x 700 8.7 / 8.3, 800 x 700
+// 9.0 / 9.1; FP16 640 x 640 8.8 / 8.1, 700 x 700 9.2 / 9.8. With a body force
+// through 15% of solids, where every node takes the general form, the node kernel
+// gains more and farther: FP32 640 x 640 10.0 / 7.9, 1001 x 701 15.4 / 12.2, 1400
+// x 1000 30.1 / 28.2; FP16 640 x 640 10.7 / 9.0, 700 x 700 11.6 / 10.9, 800 x 700
+// 11.8 / 12.1 (5 or 30% alike; BF16 as FP16); the line does not use that. FP64
+// gains at every size measured, up to 4096 x 1024.
 bool nodewise_rule(const vplbm_config* c) {
   const int rows = tile_rows_of(c) / warps_per_block(c->storage);
   if (tile_x(c->storage) * rows > kNodeThreads) return false;

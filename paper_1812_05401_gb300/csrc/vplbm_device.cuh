@@ -475,7 +475,7 @@ __device__ __forceinline__ T pair_d(const Consts<T>& c, T ha, T hb, int k) {
 // bits, which computes the same values through zero terms; kFree rounds the
 // collision's last products in another order. Which of the two a node takes
 // depends on its place alone (free_form), not on the kernel.
-// REF: h holds the elements e = h - h_ref of a 16-bit store.
+// REF: h holds the stored elements of a 16-bit (h - h_ref) or FP64 (h + w) store.
 enum { kGeneral = 0, kFluid = 1, kFree = 2 };
 
 template <class T, int FORM = kGeneral, bool REF = false>
@@ -536,9 +536,11 @@ __device__ __forceinline__ Macro<T> macros(const StepParams& p, const T h[9], ui
 // K = s+ (drho - 1.5 rho u.u) - 3 (1 - s+/2) u.F. SRT with Eq. Guo1 is the
 // same with s+ = s- = 1/tau. This is the moment-space operator rearranged,
 // not an approximation of it.
-// On the elements e = h - r of a 16-bit store (REF) the update is the same,
-// e*_a = e_a + P + Q, with d decoded from the elements (pair_d); r is odd in
-// xi, so s, e_0 = h_0 and the rest population's update need no decoding.
+// On stored elements (REF) the update of a pair is the same, e*_a = e_a + P + Q.
+// 16-bit: e = h - r with r odd in xi, so the pair sums s and the rest population
+// need no decoding, the differences d take the pair's constant (pair_d). FP64:
+// e = h + w with w even in xi, so d needs none, and s and the rest population
+// take the weights off (pair_s, rest_in, rest_out).
 // ---------------------------------------------------------------------------
 // w: the weight of the pair's directions.
 template <class T, int FORM>
@@ -735,8 +737,7 @@ struct EdgeLane {
   }
   __device__ __forceinline__ T value(const StepParams& p, const E* src, int x0, int y, int lane) const {
     if constexpr (!GEN) {
-      // FP64 weights: 1/9 for xi_y = 0, 1/36 for the others
-      return at ? S::in_e(at[(long long)y * p.pitch], lane % 3 == 0 ? 1 : 5) : T(0);
+      return at ? S::in_e(at[(long long)y * p.pitch], 1) : T(0);
     } else {
       const bool last = x0 + TX >= p.nx;
       if (lane >= 9 || (last ? lane >= 3 && lane < 6 : lane >= 6)) return T(0);
@@ -1029,7 +1030,8 @@ __device__ __forceinline__ typename S::E fstar_e(const StepParams& p, const type
 }
 
 // What a thread adds up for a step's record over the rows it collides: sum of
-// drho, and the force on its solid nodes (<= 16, arithmetic type).
+// drho, and the force on its solid nodes (at most 16, or 32 of a 16-bit store,
+// whose blocks have half the warps), in the arithmetic type.
 template <class T>
 struct RowSums {
   T dm = T(0), fx = T(0), fy = T(0);
@@ -1144,8 +1146,8 @@ __device__ __forceinline__ void round_words(const StepParams& p, int xb, int y, 
 }
 
 // A tile's share of a step's records (reduce_kernel adds the tiles): the force
-// on the solid nodes, summed per thread in the arithmetic type (each thread
-// holds at most 16 nodes) and in FP64 from the thread up; the total density, in
+// on the solid nodes, summed per thread in the arithmetic type (at most 16 nodes,
+// or 32 of a 16-bit store) and in FP64 from the thread up; the total density, in
 // the arithmetic type within the block and FP64 from the tile up. Warps and
 // blocks without solid nodes skip the FP64 work (on GB300 FP64 runs at a small
 // fraction of the FP32 rate).

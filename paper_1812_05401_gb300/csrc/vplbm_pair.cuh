@@ -14,12 +14,13 @@ namespace vplbm {
 // single step's code in its order: two steps here give the bits of two single
 // steps.
 //
-// A single step is bound by HBM (16384 x 4096: 0.773 ms with the mask's update,
-// 74 bytes a node); this kernel moves half the bytes and is bound by instruction
-// issue and latency at 24 warps an SM (IPC 1.95). Per step, single against pair:
-// 16384 x 4096 773 -> 625 us, 4096 x 1024 51.7 -> 45.2, 6048 x 2016 (SRT,
-// convective) 150 -> 133. What it took, on 16384 x 4096 (us a step, tiles of one
-// part):
+// A single step is bound by HBM (16384 x 4096: 0.734 ms, 73 bytes a node); this
+// kernel moves half the bytes and is bound by instruction issue and latency at 24
+// warps an SM (IPC 1.95). Per step of long calls, single against pair: 16384 x
+// 4096 734 -> 578 us, 4096 x 1024 49.4 -> 43.1, 6048 x 2016 (SRT, convective)
+// 142 -> 126 (pair_rule has the line). What it took, on 16384 x 4096 with a moving
+// cylinder (us a step of batches of 20 with their mask updates and the field read
+// at the end; tiles of one part):
 // - direct loads in the first step, a row at a time: 766 (latency); the rows on
 //   their way to shared memory at once (stage): 658;
 // - a lane's nodes one after the other (collide_row's ONE): 110 registers become
@@ -27,7 +28,7 @@ namespace vplbm {
 //   at a time, 80 bytes of spills: 622);
 // - edges and masks of both rows loaded ahead: 602, not kept.
 // Tiles of 32 rows in two parts, for the order of the single step's records,
-// cost 625 against 598 as tiles of 16.
+// cost 625 against 598 as tiles of 16, on the same measure.
 //
 // Shared memory: v[a][j][TX], the populations of direction a that row j of the
 // part pulls, by the column they come from, and halo[side][k][j], those that
