@@ -148,17 +148,19 @@ typedef struct {
    * stream). When set, every device buffer the solver owns comes from
    * dev_alloc(bytes, alloc_ctx) and goes back through dev_free(ptr,
    * alloc_ctx): the populations, mask, reduction scratch and rings at
-   * vplbm_create, the solid-velocity, momentum-exchange and small grids'
-   * record buffers when first needed, and the staging buffers of host transfers. dev_alloc returns
-   * memory on the current device, aligned to 256 bytes and ready for work
-   * queued afterwards on the solver's stream (PyTorch's caching allocator on
-   * that stream qualifies), or NULL when it has none: the call then fails
-   * with VPLBM_ERR_NOMEM. A pointer that is not 256-byte aligned goes back
-   * through dev_free and the call fails with VPLBM_ERR_INVALID. The library
-   * waits for the solver's stream before every dev_free, so the allocator may
-   * hand the block out again at once; calls that stage through a temporary
-   * buffer therefore return after their device work. Both functions are
-   * called on the thread that makes the library call. vplbm_group_step's
+   * vplbm_create, the solid-velocity and momentum-exchange buffers and, in
+   * vplbm_step, small grids' record window and the second mask of paired
+   * steps when first needed, and the staging buffers of host transfers.
+   * dev_alloc returns memory on the current device, aligned to 256 bytes and
+   * ready for work queued afterwards on the solver's stream (PyTorch's caching
+   * allocator on that stream qualifies), or NULL when it has none: the call
+   * then fails with VPLBM_ERR_NOMEM. A pointer that is not 256-byte aligned
+   * goes back through dev_free and the call fails with VPLBM_ERR_INVALID.
+   * (vplbm_step does without its two buffers in both cases and goes on.) The
+   * library waits for the solver's stream before every dev_free, so the
+   * allocator may hand the block out again at once; calls that stage through a
+   * temporary buffer therefore return after their device work. Both functions
+   * are called on the thread that makes the library call. vplbm_group_step's
    * small per-call launch tables and vplbm_step_noalloc (which allocates
    * nothing) do not use the hook. */
   void* (*dev_alloc)(size_t bytes, void* ctx);
